@@ -1,6 +1,6 @@
 // Kernel templates of the spectral passes (see fft.cu for the pass
-// structure): the three fused plane/column passes for H <= 128, the per-axis
-// passes for H > 128, and their launch templates.  Each translation unit that
+// structure): the two plane passes for H <= 128, the line passes along z and
+// y, the row passes for H > 128, and their launch templates.  Each translation unit that
 // launches them includes this header (internal linkage) and instantiates the
 // grid sizes and radix plans it serves, so that the instantiations compile in
 // parallel.
@@ -26,33 +26,50 @@ __device__ __forceinline__ int neg_mod(int k) {
     else return k == 0 ? 0 : H - k;
 }
 
-// Threads of the three fused passes (H <= 128) or of the z pass (H > 128),
-// chosen so that the radix-16 or radix-8 stages hold at most two butterflies
-// per thread.
+// Threads of the plane passes, chosen so that the radix-16 or radix-8 stages
+// hold at most two butterflies per thread.
 template <int H> struct Cfg;
-template <> struct Cfg<8> { static constexpr int NT1 = 64, NT2 = 64, NT3 = 64; };
-template <> struct Cfg<16> { static constexpr int NT1 = 256, NT2 = 256, NT3 = 256; };
-template <> struct Cfg<24> { static constexpr int NT1 = 256, NT2 = 128, NT3 = 256; };
-template <> struct Cfg<32> { static constexpr int NT1 = 256, NT2 = 256, NT3 = 256; };
-template <> struct Cfg<48> { static constexpr int NT1 = 256, NT2 = 256, NT3 = 256; };
-template <> struct Cfg<64> { static constexpr int NT1 = 512, NT2 = 512, NT3 = 512; };
-template <> struct Cfg<72> { static constexpr int NT1 = 512, NT2 = 352, NT3 = 512; };
-template <> struct Cfg<96> { static constexpr int NT1 = 768, NT2 = 608, NT3 = 768; };
-// 544 = 17 warps: one radix-16 butterfly per thread for the 65 z-transforms
-template <> struct Cfg<128> { static constexpr int NT1 = 1024, NT2 = 544, NT3 = 1024; };
-// H > 128 runs the per-axis pipeline; only the z pass (over 32-column tiles)
-// takes its threads from here
-template <> struct Cfg<144> { static constexpr int NT2 = 288; };
-template <> struct Cfg<192> { static constexpr int NT2 = 384; };
-template <> struct Cfg<216> { static constexpr int NT2 = 896; };
-template <> struct Cfg<256> { static constexpr int NT2 = 512; };
-template <> struct Cfg<288> { static constexpr int NT2 = 576; };
-template <> struct Cfg<384> { static constexpr int NT2 = 768; };
-template <> struct Cfg<432> { static constexpr int NT2 = 896; };
-template <> struct Cfg<512> { static constexpr int NT2 = 1024; };
+template <> struct Cfg<8> { static constexpr int NT1 = 64, NT3 = 64; };
+template <> struct Cfg<16> { static constexpr int NT1 = 256, NT3 = 256; };
+template <> struct Cfg<24> { static constexpr int NT1 = 256, NT3 = 256; };
+template <> struct Cfg<32> { static constexpr int NT1 = 256, NT3 = 256; };
+template <> struct Cfg<48> { static constexpr int NT1 = 256, NT3 = 256; };
+template <> struct Cfg<64> { static constexpr int NT1 = 512, NT3 = 512; };
+template <> struct Cfg<72> { static constexpr int NT1 = 512, NT3 = 512; };
+template <> struct Cfg<96> { static constexpr int NT1 = 768, NT3 = 768; };
+template <> struct Cfg<128> { static constexpr int NT1 = 1024, NT3 = 1024; };
 
-// kx columns per block of the z pass: the whole padded row up to H = 128
-template <int H> constexpr int zcols() { return H <= 128 ? H / 2 + 2 : 32; }
+// Threads of the line passes (kCols lines per block) and of the row passes
+// (H > 128 and radix plan 2: kRows complex rows per block).
+template <int H> struct LineCfg;
+template <> struct LineCfg<8> { static constexpr int NT = 64, NTX = 32; };
+template <> struct LineCfg<16> { static constexpr int NT = 64, NTX = 32; };
+template <> struct LineCfg<24> { static constexpr int NT = 128, NTX = 64; };
+template <> struct LineCfg<32> { static constexpr int NT = 128, NTX = 64; };
+template <> struct LineCfg<48> { static constexpr int NT = 192, NTX = 64; };
+template <> struct LineCfg<64> { static constexpr int NT = 128, NTX = 64; };
+template <> struct LineCfg<72> { static constexpr int NT = 192, NTX = 96; };
+template <> struct LineCfg<96> { static constexpr int NT = 192, NTX = 96; };
+template <> struct LineCfg<128> { static constexpr int NT = 128, NTX = 64; };
+template <> struct LineCfg<144> { static constexpr int NT = 192, NTX = 96; };
+template <> struct LineCfg<192> { static constexpr int NT = 256, NTX = 128; };
+template <> struct LineCfg<216> { static constexpr int NT = 288, NTX = 160; };
+template <> struct LineCfg<256> { static constexpr int NT = 256, NTX = 128; };
+template <> struct LineCfg<288> { static constexpr int NT = 384, NTX = 160; };
+template <> struct LineCfg<384> { static constexpr int NT = 384, NTX = 192; };
+template <> struct LineCfg<432> { static constexpr int NT = 384, NTX = 224; };
+template <> struct LineCfg<512> { static constexpr int NT = 512, NTX = 256; };
+
+// Blocks per SM the registers of the row and line passes are set for: 64 registers a
+// thread, or 56 where that lets a third block of 384 threads share the SM.
+template <int H> constexpr int line_blocks() {
+    return 65536 / ((H == 288 || H == 384 ? 56 : 64) * LineCfg<H>::NT);
+}
+
+template <int H> constexpr int row_blocks() { return 65536 / (64 * LineCfg<H>::NTX); }
+
+constexpr int kCols = 16;   // lines per block of the line passes: 128 bytes of neighbours
+constexpr int kRows = 8;    // rows per block of the row passes
 
 template <int H> constexpr int kxp() { return H / 2 + 2; }
 // shared-memory pitch (float2) of half-spectrum rows in the inverse pass: odd,
@@ -63,7 +80,18 @@ template <int H> constexpr int rowp() { return H + 1; }
 
 __device__ __forceinline__ int signed_mode(int k, int H) { return k < H / 2 ? k : k - H; }
 
-// ---------------------------------------------------------------- I/O helpers
+// Row layout in shared memory for lines transformed along x: position p of
+// line t at t PITCH + p + p / R1.  The first stage's lanes write R1 apart (its
+// outputs j R1 + r over lanes j), which the pad spreads over the banks; the
+// stages whose lanes take consecutive lines (eight, or eight and a few more,
+// so two butterflies per 16 lanes) want a pitch of 2 mod 16.
+template <int H, int R1> struct RowAt8 {
+    static constexpr int LEN = H + H / R1;
+    static constexpr int PITCH = LEN + (18 - LEN % 16) % 16;
+    __device__ __forceinline__ int operator()(int t, int p) const { return t * PITCH + p + p / R1; }
+};
+
+// ---------------------------------------------------------------- pointwise
 // int64 (two's complement) deposit accumulator -> float, via the signed high
 // and the unsigned low 32-bit halves (the single 64-bit conversion would run
 // on the FP64 pipe).
@@ -73,25 +101,62 @@ __device__ __forceinline__ float acc_to_float(unsigned long long q) {
     return fmaf(hi, 4294967296.0f, lo);
 }
 
-// R_tau at one node: (m*, w*) and v^n.
-// um is the u of the m source: u itself, or K_sigma * u (Eq. m_reg).
-// The quotients use the hardware reciprocal (within 2 ulp): the
-// denominators are at least 1.
+// R_tau at one node (explicit Euler of S = (-alpha m v; u; gamma v - eta(u) w),
+// eta(u) = 2u/(1+u)): m*, w* and v^n.  um is the u of the m source: u itself,
+// or K_sigma * u (Eq. m_reg).  The quotients use the hardware reciprocal
+// (within 2 ulp): the denominators are at least 1.
+__device__ __forceinline__ float react_m(const SpectralArgs& a, float mm, float um) {
+    return mm + a.tau * um;
+}
+__device__ __forceinline__ float react_w(const SpectralArgs& a, float vv, float ww, float u) {
+    const float eta = __fdividef(2.0f * u, 1.0f + u);
+    return ww + a.tau * (a.gamma * vv - eta * ww);
+}
+__device__ __forceinline__ float react_v(const SpectralArgs& a, float vv, float mm) {
+    return (a.v_update == SIPF_V_IMPLICIT) ? __fdividef(vv, 1.0f + a.alpha * a.tau * mm)
+                                           : vv * (1.0f - a.alpha * a.tau * mm);
+}
+
 __device__ __forceinline__ void react(const SpectralArgs& a, float vv, float mm, float ww, float u,
                                       float um, float& ms, float& ws, float& vn) {
     ms = mm;
     ws = ww;
     if (a.do_mw) {
-        // explicit Euler of S = (-alpha m v; u; gamma v - eta(u) w), eta(u) = 2u/(1+u)
-        const float eta = __fdividef(2.0f * u, 1.0f + u);
-        ms = mm + a.tau * um;
-        ws = ww + a.tau * (a.gamma * vv - eta * ww);
+        ms = react_m(a, mm, um);
+        ws = react_w(a, vv, ww, u);
     }
-    vn = (a.v_update == SIPF_V_IMPLICIT) ? __fdividef(vv, 1.0f + a.alpha * a.tau * mm)
-                                         : vv * (1.0f - a.alpha * a.tau * mm);
+    vn = react_v(a, vv, mm);
 }
 
-// ---------------------------------------------------------------- pass 1
+// The factor of mode (qx, qy, qz) on the m (field 0) or w (field 1) spectrum.
+__device__ __forceinline__ float2 diffuse_mode(const SpectralArgs& a, int field, float q2,
+                                               float2 val) {
+    const float c = field == 0 ? a.m_c : a.w_c;
+    float f = a.diffusion == SIPF_DIFFUSION_IMPLICIT ? __fdividef(1.0f, 1.0f + c * q2)
+                                                     : expf(-c * q2);
+    if (a.filter) f *= expf(-a.inv_H0sq_2pi2 * q2);
+    val = make_float2(f * val.x, f * val.y);
+    // times r0 = hi + lo: the float32 rounding of r0 itself is compensated
+    const float hi = field == 0 ? a.m_r0_hi : a.w_r0_hi;
+    const float lo = field == 0 ? a.m_r0_lo : a.w_r0_lo;
+    return make_float2(fmaf(val.x, lo, val.x * hi), fmaf(val.y, lo, val.y * hi));
+}
+
+// i k val, zero at the Nyquist mode (q = -H/2 or H/2).
+template <int H>
+__device__ __forceinline__ float2 times_ik(float scale, int q, float2 val) {
+    const float k = (q == H / 2 || q == -H / 2) ? 0.0f : scale * static_cast<float>(q);
+    return make_float2(-k * val.y, k * val.x);
+}
+
+// The modes of two real signals x1 + i x2 from z(k) and z(-k):
+// X1(k) = (z(k) + conj z(-k))/2, X2(k) = (z(k) - conj z(-k))/(2i).
+__device__ __forceinline__ void split_modes(float2 zk, float2 zc, float2& x1, float2& x2) {
+    x1 = make_float2(0.5f * (zk.x + zc.x), 0.5f * (zk.y - zc.y));
+    x2 = make_float2(0.5f * (zk.y + zc.y), -0.5f * (zk.x - zc.x));
+}
+
+// ---------------------------------------------------------------- plane pass, forward
 // Launch-parameter batches: NB = 1 for one context's step, kMaxBatch for an
 // ensemble's runs of one grid size (the run index is a grid dimension).
 template <int H, int NB, int V>
@@ -243,94 +308,66 @@ __global__ void __launch_bounds__(Cfg<H>::NT1)
     }
 }
 
-// ---------------------------------------------------------------- pass 2
-// Block (ky, field, kx tile): forward DFT along z of the KB columns
-// [k0, k0 + KB) of the (z, ky) rows, the per-mode multiplier, inverse DFT.
+// ---------------------------------------------------------------- line pass (z)
+// Block (tile, field): kCols neighbouring columns (ky, kx) of a half spectrum,
+// in flat order over the plane: forward DFT along z, the factor, inverse DFT.
+// Field 0 M, 1 W: the implicit (or exponential) diffusion factor; 2: i k_z V
+// -> B; 3 (with the low-pass filter) the filtered V -> A.  A tile's rows are whole
+// 128-byte lines (a plane has H (H/2 + 2) columns, a multiple of 16, whatever
+// the row pitch), its 16 H complex numbers take 16 KB at H = 128, so many
+// small blocks share an SM, their loads, exchanges and stores overlap, and
+// the last wave is short.  Bound by the latency of the loads and the
+// exchanges.  One block per ky row and field of 544 threads and 68 KB before:
+// 22.9 -> 18.3 us per pass at 128^3, 152 -> 91 us at 256^3.
+template <int H> struct LineShape {
+    static constexpr int TC = H * kxp<H>() / kCols;        // tiles of one half spectrum
+    static constexpr size_t bytes = (static_cast<size_t>(H) * kCols + H) * sizeof(float2);
+    static_assert(H * kxp<H>() % kCols == 0, "whole tiles");
+};
+
 template <int H, int NB, int V>
-__global__ void __launch_bounds__(Cfg<H>::NT2)
-    k_z_multiply(const __grid_constant__ SpecBatch<NB> batch) {
-    constexpr int NT = Cfg<H>::NT2, KXP = kxp<H>(), HK = H / 2 + 1, KB = zcols<H>();
-    // batches (H <= 128: one kx tile per row) take the run from grid dimension z
-    static_assert(NB == 1 || KB >= KXP, "batched z pass needs one kx tile");
+__global__ void __launch_bounds__(LineCfg<H>::NT, line_blocks<H>())
+    k_lines_z(const __grid_constant__ SpecBatch<NB> batch, int field0) {
     const SpecRun& R = batch.run[NB == 1 ? 0 : blockIdx.z];
     const SpectralArgs& a = R.a;
-    float2* __restrict__ gM = R.specM;
-    float2* __restrict__ gW = R.specW;
-    const float2* __restrict__ gV = R.specV;
-    float2* __restrict__ gB = R.specB;
-    float2* __restrict__ gA = R.specA;
-    const float2* __restrict__ twg = R.twiddle;
-    float* __restrict__ voff = R.voff;
+    constexpr int NT = LineCfg<H>::NT, KXP = kxp<H>();
     extern __shared__ float2 sm[];
-    float2* buf = sm;             // [H (z)][KB (kx)]
-    float2* tw = buf + H * KB;
-    const int ky = blockIdx.x, field = blockIdx.y;   // 0 m, 1 w, 2 v -> i k_z V, 3 v -> filtered V
-    const int k0 = NB == 1 ? blockIdx.z * KB : 0;
+    float2* buf = sm;                          // [H][kCols]
+    float2* tw = buf + H * kCols;              // [H]
     pdl_trigger();
-    if (field < 2 && !a.do_mw) return;
-    if (field == 3 && !a.filter) return;
-    const float2* src = field == 0 ? gM : field == 1 ? gW : gV;
-    float2* dst = field == 0 ? gM : field == 1 ? gW : field == 2 ? gB : gA;
-    for (int i = threadIdx.x; i < H; i += NT) tw[i] = twg[i];
+    for (int i = threadIdx.x; i < H; i += NT) tw[i] = R.twiddle[i];
+    __syncthreads();
     pdl_wait();   // the forward pass's spectra
-    constexpr int R1 = Radix<H, V>::R1;
-    // element (column t, z) of the block's tile in a [z][ky][KXP] half spectrum
-    auto at = [ky, k0](int t, int zz) -> size_t {
-        return (static_cast<size_t>(zz) * H + ky) * KXP + k0 + t;
-    };
-    // forward z DFT, its first stage loading the columns from global memory
-    stage1_from<H, R1, KB, KB, 1, NT, -1>(buf, [=](int t, int zz) {
-        return k0 + t < KXP ? src[at(t, zz)] : make_float2(0.f, 0.f);
-    });
-    // its last stage applies the per-mode factor on the way back to shared memory
-    const int qy = signed_mode(ky, H);
-    fft_rest_sink<H, V, KB, KB, 1, NT, -1>(buf, tw, [=](int t, int kz, float2 val) {
-        const int qx = k0 + t;
-        if (qx < HK) {
-            if (field == 2 && ky == 0 && qx == 0 && kz == 0) {
-                // DC of (v^n - c0): move the offset to the mean of v^n for the next step
-                *voff = *voff + val.x * a.out_scale;
-            }
+    const int field = field0 + blockIdx.y;
+    const int col = blockIdx.x * kCols + threadIdx.x % kCols;
+    const int ky = col / KXP, qx = col % KXP, qy = signed_mode(ky, H);
+    const float2* src = (field == 0 ? R.specM : field == 1 ? R.specW : R.specV) + col;
+    float2* dst = (field == 0 ? R.specM : field == 1 ? R.specW
+                  : field == 2 ? R.specB : R.specA) + col;
+    const int q2xy = qx * qx + qy * qy;
+    float* voff = R.voff;
+    round_trip<H, V, kCols, NT>(
+        buf, tw, Strided<1, kCols>{},
+        [=](int, int zz) { return src[static_cast<size_t>(zz) * (H * KXP)]; },
+        [=](int, int kz, float2 val) {
             const int qz = signed_mode(kz, H);
-            const float q2 = static_cast<float>(qx * qx + qy * qy + qz * qz);
-            float f = 1.0f;
+            const float q2 = static_cast<float>(q2xy + qz * qz);
+            if (field < 2) return diffuse_mode(a, field, q2, val);
             if (field == 2) {
-                const float kz_phys =
-                    (qz == -H / 2) ? 0.0f : a.two_pi_over_L * static_cast<float>(qz);
-                val = make_float2(-kz_phys * val.y, kz_phys * val.x);
-            } else if (field < 2) {
-                const float c = field == 0 ? a.m_c : a.w_c;
-                f = a.diffusion == SIPF_DIFFUSION_IMPLICIT ? __fdividef(1.0f, 1.0f + c * q2)
-                                                           : expf(-c * q2);
+                // DC of (v^n - c0): move the offset to the mean of v^n for the next step
+                if (col == 0 && kz == 0) *voff = *voff + val.x * a.out_scale;
+                val = times_ik<H>(a.two_pi_over_L, qz, val);
             }
-            if (a.filter) f *= expf(-a.inv_H0sq_2pi2 * q2);
-            val = make_float2(f * val.x, f * val.y);
-            if (field < 2) {
-                // times r0 = hi + lo: the float32 rounding of r0 itself is compensated
-                const float hi = field == 0 ? a.m_r0_hi : a.w_r0_hi;
-                const float lo = field == 0 ? a.m_r0_lo : a.w_r0_lo;
-                val = make_float2(fmaf(val.x, lo, val.x * hi), fmaf(val.y, lo, val.y * hi));
+            if (a.filter) {
+                const float f = expf(-a.inv_H0sq_2pi2 * q2);
+                val = make_float2(f * val.x, f * val.y);
             }
-        }
-        buf[kz * KB + t] = val;
-    });
-    // inverse z DFT, its last stage storing the columns to global memory
-    stage<H, R1, 1, KB, KB, 1, NT, +1>(buf, tw);
-    fft_rest_sink<H, V, KB, KB, 1, NT, +1>(buf, tw, [=](int t, int zz, float2 val) {
-        if (k0 + t < KXP) dst[at(t, zz)] = val;
-    });
+            return val;
+        },
+        [=](int, int zz, float2 val) { dst[static_cast<size_t>(zz) * (H * KXP)] = val; });
 }
 
-// Shapes of the lane-group transforms of the warp pipeline (below): P lanes
-// per line; exchange tiles of PITCH float2 per row and TILE float2 per group,
-// chosen so that the exchanges are free of bank conflicts.
-template <int H> struct LaneShape;
-template <> struct LaneShape<64> { static constexpr int P = 8, PITCH = 9, TILE = 72; };
-template <> struct LaneShape<128> { static constexpr int P = 8, PITCH = 18, TILE = 145; };
-template <> struct LaneShape<256> { static constexpr int P = 16, PITCH = 17, TILE = 272; };
-constexpr int kLaneWarps = 8;   // warps per block of the warp pipeline
-
-// ---------------------------------------------------------------- pass 3
+// ---------------------------------------------------------------- plane pass, inverse
 // Build the full-length complex row Z[kx] = X1[kx] + i X2[kx] of two real
 // signals from their half spectra (Hermitian extension, C2R semantics at
 // kx = 0 and kx = H/2).
@@ -471,614 +508,324 @@ __global__ void __launch_bounds__(Cfg<H>::NT3)
     }
 }
 
-// ---------------------------------------------------------------- warp per-axis pipeline
-// For the grid sizes with a LaneShape the whole spectral step can run as
-// five passes over lines held in registers by groups of P lanes (WarpFFT),
-// with the half spectra in global memory (L2) between them and no block
-// barrier inside a transform:
-//   wx_forward: row pairs (z, y), (z, y + H/2): reaction; m* + i w* per row
-//               and v^n of the two rows as one complex row, x DFT, split into
-//               half rows -> M, W, V
-//   wy (SIGN -1): columns (z, kx) of M, W, V: y DFT in place
-//   z:          the block z pass (k_z_multiply; its tiles read whole rows)
-//   wy (SIGN +1): columns of M, W, B in place, V (or its filtered copy) ->
-//               i k_x V, i k_y V
-//   wx_inverse: rows: (m, w), (dv/dx, dv/dy), and dv/dz row pairs, packed
-//               two real outputs per complex row, inverse x DFT; a block
-//               writes whole rows of the gather array.
-// Lines are assigned to groups in a flat order, so that a warp's groups read
-// and write neighbouring memory.
-
-// Split a transformed complex row X = X1 + i X2 of two real rows, held in
-// the spectral layout, into their half rows (kx < H/2 + 2, the last one the
-// zero padding): X1(k) = (X(k) + conj X(-k))/2, X2(k) = (X(k) - conj X(-k))/(2i).
-template <int H, class F>
-__device__ __forceinline__ void split_store(const float2 (&v)[F::Q], int l, float2* ex,
-                                            float2* d1, float2* d2) {
-    constexpr int P = F::Q / F::S, S = F::S, Q = F::Q, KXP = kxp<H>(), HK = H / 2 + 1;
-    __syncwarp();
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-#pragma unroll
-        for (int k2 = 0; k2 < P; ++k2) ex[S * l + s + Q * k2] = v[s * P + k2];
+// X1 + i X2 of two real signals at mode k from their half spectra a(k') and
+// b(k') at k' = min(k, H - k) (C2R semantics at k = 0 and k = H/2).
+template <int H>
+__device__ __forceinline__ float2 pack_modes(float2 a, float2 b, int k) {
+    if (k > H / 2) {
+        a.y = -a.y;
+        b.y = -b.y;
+    } else if (k == 0 || k == H / 2) {
+        a.y = 0.f;
+        b.y = 0.f;
     }
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < (KXP + P - 1) / P; ++j) {
-        const int k = l + P * j;
-        if (k < KXP) {
-            float2 a1 = make_float2(0.f, 0.f), a2 = a1;
-            if (k < HK) {
-                const float2 zp = ex[k], zm = ex[neg_mod<H>(k)];
-                a1 = make_float2(0.5f * (zp.x + zm.x), 0.5f * (zp.y - zm.y));
-                a2 = make_float2(0.5f * (zp.y + zm.y), -0.5f * (zp.x - zm.x));
-            }
-            d1[k] = a1;
-            if (d2) d2[k] = a2;
-        }
-    }
+    return make_float2(a.x - b.y, a.y + b.x);
 }
 
-template <int H, int NB>
-__global__ void __launch_bounds__(32 * kLaneWarps)
-    k_wx_forward(const __grid_constant__ SpecBatch<NB> batch) {
-    using C = LaneShape<H>;
-    using F = WarpFFT<H, C::P, C::PITCH>;
-    constexpr int P = C::P, Q = F::Q, G = 32 / P, KXP = kxp<H>(), HH = H / 2;
-    __shared__ float2 tw[H];
-    __shared__ float2 exch[kLaneWarps][G * C::TILE];
-    const SpecRun& R = batch.run[NB == 1 ? 0 : blockIdx.z];
-    const SpectralArgs& a = R.a;
-    for (int i = threadIdx.x; i < H; i += blockDim.x) tw[i] = R.twiddle[i];
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int g = lane / P, l = lane % P;
-    const int task = (blockIdx.x * kLaneWarps + warp) * G + g;   // (z, y < H/2)
-    if (task >= H * HH) return;    // whole groups; H * H/2 is a multiple of every group count
-    const int z = task / HH, y = task % HH;
-    float2* ex = &exch[warp][g * C::TILE];
-    const float u_scale = R.sc->u_scale;   // u_bar per accumulator unit
-    const float c0 = *R.voff;   // the v spectrum only feeds derivatives: remove a constant
-    const size_t row0 = (static_cast<size_t>(z) * H + y) * H;
-    const size_t row1 = row0 + static_cast<size_t>(HH) * H;
-    const float gamma_v = a.alpha * a.tau;
-    {
-        // v^n of the two rows as one complex row (reads v and m only)
-        float2 zv[Q];
-#pragma unroll
-        for (int m = 0; m < Q; ++m) {
-            const int x = l + P * m;
-            float vn[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const size_t o = (h ? row1 : row0) + x;
-                const float vv = R.v[o], mm = R.m[o];
-                vn[h] = (a.v_update == SIPF_V_IMPLICIT) ? __fdividef(vv, 1.0f + gamma_v * mm)
-                                                        : vv * (1.0f - gamma_v * mm);
-            }
-            zv[m] = make_float2(vn[0] - c0, vn[1] - c0);
-        }
-        F::template to_spectral<-1>(zv, l, ex, tw);
-        const size_t s0 = (static_cast<size_t>(z) * H + y) * KXP;
-        split_store<H, F>(zv, l, ex, R.specV + s0, R.specV + s0 + static_cast<size_t>(HH) * KXP);
-    }
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-        // the reaction on row y + h H/2: m* + i w*, v^n, the accumulator cleared
-        const size_t row = h ? row1 : row0;
-        float2 zr[Q];
-        // chunks of CH elements: all loads of a chunk before its stores (the
-        // stores may alias later loads, so they would otherwise wait)
-        constexpr int CH = 4;
-#pragma unroll
-        for (int m0 = 0; m0 < Q; m0 += CH) {
-            float vv[CH], mm[CH], ww[CH], uu[CH];
-            unsigned long long qq[CH];
-#pragma unroll
-            for (int c = 0; c < CH; ++c) {
-                const size_t o = row + l + P * (m0 + c);
-                vv[c] = R.v[o];
-                mm[c] = R.m[o];
-                ww[c] = R.w[o];
-                qq[c] = R.acc[o];
-                uu[c] = R.us ? R.us[o] : 0.f;
-            }
-#pragma unroll
-            for (int c = 0; c < CH; ++c) {
-                const size_t o = row + l + P * (m0 + c);
-                R.acc[o] = 0ull;
-                const float u = acc_to_float(qq[c]) * u_scale;
-                float ms, ws, vn;
-                react(a, vv[c], mm[c], ww[c], u, R.us ? uu[c] : u, ms, ws, vn);
-                zr[m0 + c] = make_float2(ms, ws);
-                if (a.write_v) R.v_out[o] = vn;
-            }
-        }
-        if (a.do_mw) {
-            F::template to_spectral<-1>(zr, l, ex, tw);
-            const size_t s = (static_cast<size_t>(z) * H + y + h * HH) * KXP;
-            split_store<H, F>(zr, l, ex, R.specM + s, R.specW + s);
-        }
-    }
-}
-
-// y DFT of columns (z, kx) of the half spectra.  SIGN -1: M, W, V in place
-// (spatial layout in, spectral out).  SIGN +1: M, W, B in place, and V (or
-// its filtered copy) -> i k_x V, i k_y V (spectral layout in, spatial out).
-template <int H, int SIGN, int NB>
-__global__ void __launch_bounds__(32 * kLaneWarps) k_wy(const __grid_constant__ SpecBatch<NB> batch) {
-    using C = LaneShape<H>;
-    using F = WarpFFT<H, C::P, C::PITCH>;
-    constexpr int P = C::P, Q = F::Q, S = F::S, G = 32 / P, KXP = kxp<H>();
-    __shared__ float2 tw[H];
-    __shared__ float2 exch[kLaneWarps][G * C::TILE];
-    const SpecRun& R = batch.run[NB == 1 ? 0 : blockIdx.z];
-    const SpectralArgs& a = R.a;
-    const int field = blockIdx.y;   // 0 M, 1 W, 2 V or B, 3 -> i k_x V, 4 -> i k_y V
-    if (field < 2 && !a.do_mw) return;
-    for (int i = threadIdx.x; i < H; i += blockDim.x) tw[i] = R.twiddle[i];
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int g = lane / P, l = lane % P;
-    const int col = (blockIdx.x * kLaneWarps + warp) * G + g;   // (z, kx)
-    if (col >= H * KXP) return;    // whole groups
-    const int z = col / KXP, kx = col % KXP;
-    float2* ex = &exch[warp][g * C::TILE];
-    const float2* vsrc = a.filter ? R.specA : R.specV;
-    const float2* src = field == 0 ? R.specM : field == 1 ? R.specW
-                      : field == 2 ? (SIGN < 0 ? R.specV : R.specB) : vsrc;
-    float2* dst = field == 0 ? R.specM : field == 1 ? R.specW
-                : field == 2 ? (SIGN < 0 ? R.specV : R.specB) : field == 3 ? R.specDx : R.specDy;
-    const size_t base = static_cast<size_t>(z) * H * KXP + kx;
-    float2 v[Q];
-    if constexpr (SIGN < 0) {
-#pragma unroll
-        for (int m = 0; m < Q; ++m) v[m] = src[base + static_cast<size_t>(l + P * m) * KXP];
-        F::template to_spectral<-1>(v, l, ex, tw);
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-#pragma unroll
-            for (int k2 = 0; k2 < P; ++k2)
-                dst[base + static_cast<size_t>(S * l + s + Q * k2) * KXP] = v[s * P + k2];
-        }
-    } else {
-        const float kxs_ = (kx >= H / 2) ? 0.0f : a.two_pi_over_L * static_cast<float>(kx);
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-#pragma unroll
-            for (int k2 = 0; k2 < P; ++k2) {
-                const int ky = S * l + s + Q * k2;
-                float2 val = src[base + static_cast<size_t>(ky) * KXP];
-                if (field >= 3) {
-                    float k;
-                    if (field == 3) {
-                        k = kxs_;
-                    } else {
-                        const int qy = signed_mode(ky, H);
-                        k = (qy == -H / 2) ? 0.0f : a.two_pi_over_L * static_cast<float>(qy);
-                    }
-                    val = make_float2(-k * val.y, k * val.x);
-                }
-                v[s * P + k2] = val;
-            }
-        }
-        F::template to_spatial<+1>(v, l, ex, tw);
-#pragma unroll
-        for (int m = 0; m < Q; ++m) dst[base + static_cast<size_t>(l + P * m) * KXP] = v[m];
-    }
-}
-
-// Inverse x DFT of packed rows: (m, w) rows, (dv/dx, dv/dy) rows and dv/dz
-// row pairs (y, y + H/2); scaled outputs.  A block takes PB row pairs
-// (y0 + t, y0 + t + H/2), t < PB, of one plane: 2 PB (m, w) rows, 2 PB
-// (dv/dx, dv/dy) rows and PB dv/dz pairs, each warp of one kind, so that the
-// four components of each node of the gather array are written close
-// together in time (they are written by three kinds of tasks).
-template <int H> struct WxInv {
-    static constexpr int G = 32 / LaneShape<H>::P;          // lines per warp
-    static constexpr int PB = 2 * G;                        // row pairs per block
-    static constexpr int WMW = 2 * PB / G, WD = 2 * PB / G, WB = PB / G;
-    static constexpr int WARPS = WMW + WD + WB;             // 10
+// ---------------------------------------------------------------- line pass (y)
+// For the per-axis pipeline: y DFT of kCols lines of the half spectra.  Tiles
+// of kCols neighbouring columns kx < H/2 of one plane, then tiles of the kx =
+// H/2 columns of kCols planes (which would otherwise cost every plane a tile
+// of one column).  SIGN -1: families 0 M, 1 W, 2 V in place.  SIGN +1: 0
+// M, 1 W, 2 B in place, V (or its filtered copy) -> 3 i k_x V, 4 i k_y V.
+template <int H> struct YTiles {
+    static constexpr int PER = (H / 2 + kCols - 1) / kCols;             // per plane
+    static constexpr int ALL = H * PER + (H + kCols - 1) / kCols;
 };
 
-template <int H, int NB>
-__global__ void __launch_bounds__(32 * WxInv<H>::WARPS)
-    k_wx_inverse(const __grid_constant__ SpecBatch<NB> batch) {
-    using C = LaneShape<H>;
-    using F = WarpFFT<H, C::P, C::PITCH>;
-    using X = WxInv<H>;
-    constexpr int P = C::P, Q = F::Q, S = F::S, G = X::G, PB = X::PB, KXP = kxp<H>(), HH = H / 2;
-    static_assert(HH % PB == 0, "whole blocks of row pairs");
-    __shared__ float2 tw[H];
-    __shared__ float2 exch[X::WARPS][G * C::TILE];
-    const SpecRun& R = batch.run[NB == 1 ? 0 : blockIdx.z];
-    const SpectralArgs& a = R.a;
-    for (int i = threadIdx.x; i < H; i += blockDim.x) tw[i] = R.twiddle[i];
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int g = lane / P, l = lane % P;
-    constexpr int YB = HH / PB;                     // blocks of PB row pairs per plane
-    const int z = blockIdx.x / YB, y0 = (blockIdx.x % YB) * PB;
-    int kind, y;
-    if (warp < X::WMW) {
-        kind = 0;
-        const int t = warp * G + g;                 // 0 .. 2 PB - 1
-        y = y0 + (t % PB) + (t / PB) * HH;
-    } else if (warp < X::WMW + X::WD) {
-        kind = 1;
-        const int t = (warp - X::WMW) * G + g;
-        y = y0 + (t % PB) + (t / PB) * HH;
-    } else {
-        kind = 2;
-        y = y0 + (warp - X::WMW - X::WD) * G + g;   // pair (y, y + H/2)
-    }
-    if (kind == 0 && !a.do_mw) return;              // whole warps
-    float2* ex = &exch[warp][g * C::TILE];
-    const size_t r0 = (static_cast<size_t>(z) * H + y) * KXP;
-    const float2* p1;
-    const float2* p2;
-    if (kind == 0) {
-        p1 = R.specM + r0;
-        p2 = R.specW + r0;
-    } else if (kind == 1) {
-        p1 = R.specDx + r0;
-        p2 = R.specDy + r0;
-    } else {
-        p1 = R.specB + r0;
-        p2 = R.specB + r0 + static_cast<size_t>(HH) * KXP;
-    }
-    float2 v[Q];
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-#pragma unroll
-        for (int k2 = 0; k2 < P; ++k2) v[s * P + k2] = pack_two<H>(p1, p2, S * l + s + Q * k2);
-    }
-    F::template to_spatial<+1>(v, l, ex, tw);
-    const size_t node0 = (static_cast<size_t>(z) * H + y) * H;
-    if (kind == 0) {
-        const float sc = a.out_scale;
-#pragma unroll
-        for (int m = 0; m < Q; ++m) {
-            const size_t node = node0 + l + P * m;
-            const float wv = v[m].y * sc;
-            R.m_out[node] = v[m].x * sc;
-            R.w_out[node] = wv;
-            R.G[4 * node + 3] = wv;
-        }
-    } else if (kind == 1) {
-        const float sxy = a.out_scale_xy;
-#pragma unroll
-        for (int m = 0; m < Q; ++m) {
-            const size_t node = node0 + l + P * m;
-            *reinterpret_cast<float2*>(R.G + 4 * node) = make_float2(v[m].x * sxy, v[m].y * sxy);
-        }
-    } else {
-        const float sc = a.out_scale;
-        const size_t node1 = node0 + static_cast<size_t>(HH) * H;
-#pragma unroll
-        for (int m = 0; m < Q; ++m) {
-            R.G[4 * (node0 + l + P * m) + 2] = v[m].x * sc;
-            R.G[4 * (node1 + l + P * m) + 2] = v[m].y * sc;
-        }
-    }
-}
-
-// Blocks covering n lines (groups of 32 / P lanes in kLaneWarps warps).
-template <int H> constexpr int warp_blocks(int n) {
-    constexpr int per_block = kLaneWarps * (32 / LaneShape<H>::P);
-    return (n + per_block - 1) / per_block;
-}
-
-// The warp pipeline's passes, grouped like the fused ones.
-template <int H, int NB>
-cudaError_t warp_pass(const SpecBatch<NB>& batch, int nb, int pass, int device, cudaStream_t s) {
-    constexpr int KXP = kxp<H>(), NT = 32 * kLaneWarps, KB = zcols<H>();
-    constexpr size_t smz = (static_cast<size_t>(H) * KB + H) * sizeof(float2);
-    static int configured_device = -1;
-    if (configured_device != device) {
-        cudaFuncSetAttribute(k_z_multiply<H, NB, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(smz));
-        configured_device = device;
-    }
-    if (pass == 0) {
-        k_wx_forward<H, NB><<<dim3(warp_blocks<H>(H * (H / 2)), 1, nb), NT, 0, s>>>(batch);
-        k_wy<H, -1, NB><<<dim3(warp_blocks<H>(H * KXP), 3, nb), NT, 0, s>>>(batch);
-    } else if (pass == 1) {
-        k_z_multiply<H, NB, 0><<<dim3(H, 4, NB == 1 ? (KXP + KB - 1) / KB : nb), Cfg<H>::NT2, smz,
-                                 s>>>(batch);
-    } else {
-        k_wy<H, +1, NB><<<dim3(warp_blocks<H>(H * KXP), 5, nb), NT, 0, s>>>(batch);
-        k_wx_inverse<H, NB><<<dim3(H * (H / 2 / WxInv<H>::PB), 1, nb), 32 * WxInv<H>::WARPS, 0,
-                              s>>>(batch);
-    }
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------- per-axis passes (H > 128)
-// A plane above 128^2 does not fit in shared memory, so for H > 128 each
-// axis is transformed by its own kernel over small blocks of lines:
-//   sx_forward: rows of RB lines: reaction, x DFT (row pairs) -> half spectra
-//   sx_columns: columns (KB kx at a time) of one plane: y DFT, forward or
-//               inverse; in the inverse, V becomes i k_x V and i k_y V
-//   k_z_multiply (32-column tiles) between them, then
-//   sx_inverse: rows: pack two real outputs per complex row, inverse x DFT.
-constexpr int kSxRows = 8;     // rows per block of the x passes
-constexpr int kSxCols = 16;    // kx columns per block of the y passes
-constexpr int kSxNT = 256;
-
-template <int H, int V>
-__global__ void __launch_bounds__(kSxNT)
-    k_sx_forward(SpectralArgs a, const float* v, const float* __restrict__ m,
-                 const float* __restrict__ w, unsigned long long* __restrict__ acc, float* v_out,
-                 float2* __restrict__ gM, float2* __restrict__ gW, float2* __restrict__ gV,
-                 const float2* __restrict__ twg, const float* __restrict__ voff,
-                 const StepScalars* __restrict__ sc, const float* __restrict__ us) {
-    constexpr int RB = kSxRows, NT = kSxNT, KXP = kxp<H>(), HK = H / 2 + 1, RP = rowp<H>();
-    const float u_scale = sc->u_scale;   // u_bar per accumulator unit
-    static_assert((RB / 2) * RP <= RB * KXP, "row pairs fit in the half-row space");
-    extern __shared__ float2 sm[];
-    float2* buf = sm;              // 3 fields: [RB/2][RP] row pairs, then [RB][KXP] half rows
-    float2* tw = buf + 3 * RB * KXP;
-    const int z = blockIdx.y, y0 = blockIdx.x * RB;
-    for (int i = threadIdx.x; i < H; i += NT) tw[i] = twg[i];
-    const float c0 = *voff;
-    const size_t row0 = (static_cast<size_t>(z) * H + y0) * H;
-    for (int g = threadIdx.x; g < RB * H / 4; g += NT) {
-        const size_t o = row0 + 4 * static_cast<size_t>(g);
-        const float4 rv = *reinterpret_cast<const float4*>(v + o);
-        const float4 rm = *reinterpret_cast<const float4*>(m + o);
-        const float4 rw = *reinterpret_cast<const float4*>(w + o);
-        const ulonglong2 q0 = *reinterpret_cast<const ulonglong2*>(acc + o);
-        const ulonglong2 q1 = *reinterpret_cast<const ulonglong2*>(acc + o + 2);
-        *reinterpret_cast<ulonglong2*>(acc + o) = make_ulonglong2(0ull, 0ull);
-        *reinterpret_cast<ulonglong2*>(acc + o + 2) = make_ulonglong2(0ull, 0ull);
-        const float vv[4] = {rv.x, rv.y, rv.z, rv.w}, mm[4] = {rm.x, rm.y, rm.z, rm.w};
-        const float ww[4] = {rw.x, rw.y, rw.z, rw.w};
-        const unsigned long long qq[4] = {q0.x, q0.y, q1.x, q1.y};
-        const int r = (4 * g) / H, x0 = (4 * g) % H;
-        float vn[4];
-        float4 ru = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (us) ru = *reinterpret_cast<const float4*>(us + o);
-        const float uu[4] = {ru.x, ru.y, ru.z, ru.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            float ms, ws;
-            const float u = acc_to_float(qq[e]) * u_scale;
-            react(a, vv[e], mm[e], ww[e], u, us ? uu[e] : u, ms, ws, vn[e]);
-            const float val[3] = {ms, ws, vn[e] - c0};
-#pragma unroll
-            for (int f = 0; f < 3; ++f)
-                reinterpret_cast<float*>(buf + (f * (RB / 2) + (r >> 1)) * RP)[2 * (x0 + e) + (r & 1)] =
-                    val[f];
-        }
-        if (a.write_v) *reinterpret_cast<float4*>(v_out + o) = make_float4(vn[0], vn[1], vn[2], vn[3]);
-    }
-    __syncthreads();
-    fft_axis<H, V, 3 * (RB / 2), 1, RP, NT, -1>(buf, tw);
-    {
-        // split each transformed row pair into the two rows' half spectra
-        constexpr int NS = 3 * (RB / 2) * HK, SPT = (NS + NT - 1) / NT;
-        float2 x1[SPT], x2[SPT];
-#pragma unroll
-        for (int t = 0; t < SPT; ++t) {
-            const int idx = threadIdx.x + t * NT;
-            if (idx < NS) {
-                const int pr = idx / HK, k = idx % HK;
-                const float2 zp = buf[pr * RP + k];
-                const float2 zm = buf[pr * RP + neg_mod<H>(k)];
-                x1[t] = make_float2(0.5f * (zp.x + zm.x), 0.5f * (zp.y - zm.y));
-                x2[t] = make_float2(0.5f * (zp.y + zm.y), -0.5f * (zp.x - zm.x));
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int t = 0; t < SPT; ++t) {
-            const int idx = threadIdx.x + t * NT;
-            if (idx < NS) {
-                const int pr = idx / HK, k = idx % HK;
-                const int f = pr / (RB / 2), p = pr % (RB / 2);
-                buf[(f * RB + 2 * p) * KXP + k] = x1[t];
-                buf[(f * RB + 2 * p + 1) * KXP + k] = x2[t];
-            }
-        }
-        __syncthreads();
-    }
-    for (int q = threadIdx.x; q < 3 * RB * (KXP / 2); q += NT) {
-        const int f = q / (RB * (KXP / 2)), rem = q % (RB * (KXP / 2));
-        const int r = rem / (KXP / 2), k = 2 * (rem % (KXP / 2));
-        if (f < 2 && !a.do_mw) continue;
-        float2* dst = f == 0 ? gM : f == 1 ? gW : gV;
-        const float2 e0 = buf[(f * RB + r) * KXP + k];
-        const float2 e1 = k + 1 < HK ? buf[(f * RB + r) * KXP + k + 1] : make_float2(0.f, 0.f);
-        *reinterpret_cast<float4*>(dst + (static_cast<size_t>(z) * H + y0 + r) * KXP + k) =
-            make_float4(e0.x, e0.y, e1.x, e1.y);
-    }
-}
-
-// y DFT of KB kx columns of one plane of `field` (forward: M, W, V in place;
-// inverse: M, W, B in place, and V (or its filtered copy) -> i k_x V, i k_y V).
 template <int H, int SIGN, int V>
-__global__ void __launch_bounds__(kSxNT)
-    k_sx_columns(SpectralArgs a, float2* f0, float2* f1, float2* f2, float2* __restrict__ dx,
-                 float2* __restrict__ dy,
-                 const float2* __restrict__ twg, int plain) {
-    constexpr int NT = kSxNT, KXP = kxp<H>(), KB = kSxCols, CP = KB + 1;
+__global__ void __launch_bounds__(LineCfg<H>::NT)
+    k_lines_y(const __grid_constant__ SpecBatch<1> batch, int family0) {
+    const SpecRun& R = batch.run[0];
+    const SpectralArgs& a = R.a;
+    constexpr int NT = LineCfg<H>::NT, KXP = kxp<H>(), HH = H / 2, PER = YTiles<H>::PER;
     extern __shared__ float2 sm[];
-    float2* tw = sm;               // [H]
-    float2* b0 = tw + H;           // [H (y)][CP]
-    float2* b1 = b0 + H * CP;      // second buffer (derivatives; allocated only for them)
-    const int k0 = blockIdx.x * KB, z = blockIdx.y, field = blockIdx.z;
-    if (!plain && field < 2 && !a.do_mw) return;
-    const bool deriv = !plain && SIGN > 0 && field == 2;
-    float2* src = field == 0 ? f0 : field == 1 ? f1 : f2;
-    for (int i = threadIdx.x; i < H; i += NT) tw[i] = twg[i];
-    const size_t plane = static_cast<size_t>(z) * H * KXP;
-    for (int q = threadIdx.x; q < H * KB; q += NT) {
-        const int y = q / KB, t = q % KB, k = k0 + t;
-        float2 val = k < KXP ? src[plane + static_cast<size_t>(y) * KXP + k] : make_float2(0.f, 0.f);
-        if (deriv) {
-            const int qy = signed_mode(y, H);
-            const float kxp_ = (k >= H / 2) ? 0.0f : a.two_pi_over_L * static_cast<float>(k);
-            const float kyp = (qy == -H / 2) ? 0.0f : a.two_pi_over_L * static_cast<float>(qy);
-            b1[y * CP + t] = make_float2(-kyp * val.y, kyp * val.x);
-            val = make_float2(-kxp_ * val.y, kxp_ * val.x);
-        }
-        b0[y * CP + t] = val;
-    }
+    float2* buf = sm;
+    float2* tw = buf + H * kCols;
+    for (int i = threadIdx.x; i < H; i += NT) tw[i] = R.twiddle[i];
     __syncthreads();
-    fft_axis<H, V, KB, CP, 1, NT, SIGN>(b0, tw);
-    if (deriv) fft_axis<H, V, KB, CP, 1, NT, SIGN>(b1, tw);
-    float2* d0 = deriv ? dx : src;
-    for (int q = threadIdx.x; q < H * KB; q += NT) {
-        const int y = q / KB, t = q % KB, k = k0 + t;
-        if (k >= KXP) continue;
-        d0[plane + static_cast<size_t>(y) * KXP + k] = b0[y * CP + t];
-        if (deriv) dy[plane + static_cast<size_t>(y) * KXP + k] = b1[y * CP + t];
-    }
-}
-
-// Rows of the inverse: (m, w), (dv/dx, dv/dy) and dv/dz row pairs, packed
-// two real outputs per complex row, inverse x DFT, scaled outputs.
-template <int H, int V>
-__global__ void __launch_bounds__(kSxNT)
-    k_sx_inverse(SpectralArgs a, const float2* __restrict__ gM, const float2* __restrict__ gW,
-                 const float2* __restrict__ gDx, const float2* __restrict__ gDy,
-                 const float2* __restrict__ gB, float* __restrict__ m_out,
-                 float* __restrict__ w_out, float* __restrict__ G, const float2* __restrict__ twg) {
-    constexpr int RB = kSxRows, NT = kSxNT, KXP = kxp<H>(), RP = rowp<H>();
-    constexpr int NZ = RB + RB + RB / 2;       // packed rows: (m, w), (dx, dy), dz pairs
-    extern __shared__ float2 sm[];
-    float2* Z = sm;                            // [NZ][RP]
-    float2* tw = Z + NZ * RP;
-    const int z = blockIdx.y, y0 = blockIdx.x * RB;
-    for (int i = threadIdx.x; i < H; i += NT) tw[i] = twg[i];
-    // pack straight from the half spectra in global memory (consecutive lanes
-    // read consecutive, or mirrored consecutive, kx), so that the block holds
-    // only the packed rows and more blocks share an SM
-    auto row = [z, y0](const float2* f, int r) {
-        return f + (static_cast<size_t>(z) * H + y0 + r) * KXP;
-    };
-    for (int q = threadIdx.x; q < NZ * H; q += NT) {
-        const int zr = q / H, kx = q % H;
-        float2 val;
-        if (zr < RB) {
-            val = a.do_mw ? pack_two<H>(row(gM, zr), row(gW, zr), kx) : make_float2(0.f, 0.f);
-        } else if (zr < 2 * RB) {
-            const int r = zr - RB;
-            val = pack_two<H>(row(gDx, r), row(gDy, r), kx);
-        } else {
-            const int p = zr - 2 * RB;
-            val = pack_two<H>(row(gB, 2 * p), row(gB, 2 * p + 1), kx);
-        }
-        Z[zr * RP + kx] = val;
-    }
-    __syncthreads();
-    fft_axis<H, V, NZ, 1, RP, NT, +1>(Z, tw);
-    const float sc = a.out_scale, sxy = a.out_scale_xy;
-    for (int q = threadIdx.x; q < RB * H; q += NT) {
-        const int r = q / H, x = q % H;
-        const size_t node = (static_cast<size_t>(z) * H + y0 + r) * H + x;
-        const float2 mw = Z[r * RP + x];
-        const float2 dxy = Z[(RB + r) * RP + x];
-        const float2 bz = Z[(2 * RB + (r >> 1)) * RP + x];
-        if (a.do_mw) {
-            m_out[node] = mw.x * sc;
-            w_out[node] = mw.y * sc;
-            *reinterpret_cast<float4*>(G + 4 * node) =
-                make_float4(dxy.x * sxy, dxy.y * sxy, ((r & 1) ? bz.y : bz.x) * sc, mw.y * sc);
-        } else {
-            *reinterpret_cast<float2*>(G + 4 * node) = make_float2(dxy.x * sxy, dxy.y * sxy);
-            G[4 * node + 2] = ((r & 1) ? bz.y : bz.x) * sc;
-        }
-    }
-}
-
-// Passes of the per-axis pipeline, grouped like the fused ones:
-// 0 forward (x, y), 1 z, 2 inverse (y, x).
-template <int H, int V>
-cudaError_t spectral_pass_split_v(sipf_ctx* c, const SpectralArgs& a, int pass) {
-    constexpr int KXP = kxp<H>(), RB = kSxRows, KB = kSxCols, RP = rowp<H>();
-    const size_t smx1 = (3 * static_cast<size_t>(RB) * KXP + H) * sizeof(float2);
-    // the column passes: one buffer, or two where V becomes i k_x V and i k_y V
-    const size_t smy1 = (static_cast<size_t>(H) * (KB + 1) + H) * sizeof(float2);
-    const size_t smy2 = (2 * static_cast<size_t>(H) * (KB + 1) + H) * sizeof(float2);
-    const size_t smz = (static_cast<size_t>(H) * zcols<H>() + H) * sizeof(float2);
-    const size_t smx2 = (static_cast<size_t>(2 * RB + RB / 2) * RP + H) * sizeof(float2);
-    static int configured_device = -1;
-    if (configured_device != c->device) {
-        cudaFuncSetAttribute(k_sx_forward<H, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(smx1));
-        cudaFuncSetAttribute(k_sx_columns<H, -1, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(smy1));
-        cudaFuncSetAttribute(k_sx_columns<H, +1, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(smy2));
-        cudaFuncSetAttribute(k_z_multiply<H, 1, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(smz));
-        cudaFuncSetAttribute(k_sx_inverse<H, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(smx2));
-        configured_device = c->device;
-    }
-    const dim3 gy((KXP + KB - 1) / KB, H, 3);
-    if (pass == 0) {
-        k_sx_forward<H, V><<<dim3(H / RB, H), kSxNT, smx1, c->stream>>>(
-            a, c->v, c->m, c->w, reinterpret_cast<unsigned long long*>(c->acc), c->v, c->specM,
-            c->specW, c->specV, c->twiddle, c->voff, c->dsc + c->cur, c->us);
-        k_sx_columns<H, -1, V><<<gy, kSxNT, smy1, c->stream>>>(a, c->specM, c->specW, c->specV,
-                                                              nullptr, nullptr, c->twiddle, 0);
-    } else if (pass == 1) {
-        SpecBatch<1> one;
-        one.run[0] = spec_run(c, a);
-        k_z_multiply<H, 1, V><<<dim3(H, 4, (KXP + zcols<H>() - 1) / zcols<H>()), Cfg<H>::NT2, smz,
-                               c->stream>>>(one);
+    const int tile = blockIdx.x, t0 = threadIdx.x % kCols;
+    int z, k;
+    bool in;
+    if (tile < H * PER) {
+        z = tile / PER;
+        k = (tile % PER) * kCols + t0;
+        in = k < HH;
     } else {
-        // inverse y: M, W and B in place; V (or its filtered copy) -> i k_x V, i k_y V
-        k_sx_columns<H, +1, V><<<gy, kSxNT, smy2, c->stream>>>(
-            a, c->specM, c->specW, a.filter ? c->specA : c->specV, c->specDx, c->specDy, c->twiddle,
-            0);
-        k_sx_columns<H, +1, V><<<dim3(gy.x, H, 1), kSxNT, smy1, c->stream>>>(
-            a, c->specB, c->specB, c->specB, nullptr, nullptr, c->twiddle, 1);
-        k_sx_inverse<H, V><<<dim3(H / RB, H), kSxNT, smx2, c->stream>>>(
-            a, c->specM, c->specW, c->specDx, c->specDy, c->specB, c->m, c->w, c->G, c->twiddle);
+        z = (tile - H * PER) * kCols + t0;
+        k = HH;
+        in = z < H;
     }
-    return cudaGetLastError();
+    const int family = family0 + blockIdx.y;
+    const size_t base = static_cast<size_t>(z) * H * KXP + k;
+    const float2* src = (family == 0 ? R.specM : family == 1 ? R.specW
+                        : family == 2 ? (SIGN < 0 ? R.specV : R.specB)
+                        : a.filter ? R.specA : R.specV) + base;
+    float2* dst = (family == 0 ? R.specM : family == 1 ? R.specW
+                  : family == 2 ? (SIGN < 0 ? R.specV : R.specB)
+                  : family == 3 ? R.specDx : R.specDy) + base;
+    const float ks = a.two_pi_over_L;
+    one_way<H, V, kCols, NT, SIGN, false, false>(
+        buf, tw, Strided<1, kCols>{},
+        [=](int, int y) {
+            if (!in) return make_float2(0.f, 0.f);
+            float2 x = src[y * KXP];
+            if (SIGN > 0 && family >= 3)
+                x = times_ik<H>(ks, family == 3 ? k : signed_mode(y, H), x);
+            return x;
+        },
+        [=](int, int y, float2 val) {
+            if (in) dst[y * KXP] = val;
+        });
 }
 
-// Shared memory of the fused passes.
+// ---------------------------------------------------------------- row passes
+// x transforms of kRows complex rows for the per-axis pipeline.  Forward, by
+// MODE: 0 (radix plan 2) m* + i w* of kRows rows; 1 pairs of neighbouring rows
+// (2p, 2p + 1) of m*, then of w*; 2, 3 pairs of rows of v^n - c0, (2p, 2p + 1) or
+// (radix plan 2) (y, y + H/2).  Modes 0 and 1 store v^n and clear the deposit
+// accumulator; 2 and 3 follow them in a launch of their own, which reads v^n
+// again but keeps every thread busy (v^n within the first launch left half
+// the threads idle: 207 us against 128 + 24 at 256^3).  Out: the half rows (kx <= H/2)
+// of M and W, or of V.  The loads feed the first stage in registers.  Bound by
+// DRAM (60 bytes per node and 12 per mode at 256^3 and above).
+template <int H, int V> struct RowShape {
+    static constexpr int R1 = Radix<H, V>::R1;
+    using At = RowAt8<H, R1>;
+    static constexpr int Z = kRows * At::PITCH;
+    static constexpr size_t bytes = (static_cast<size_t>(Z) + H) * sizeof(float2);
+};
+
+template <int H, int V, int MODE>
+__global__ void __launch_bounds__(LineCfg<H>::NTX, row_blocks<H>())
+    k_rows_forward(const __grid_constant__ SpecBatch<1> batch) {
+    const SpecRun& R = batch.run[0];
+    const SpectralArgs& a = R.a;
+    using S = RowShape<H, V>;
+    constexpr int NT = LineCfg<H>::NTX, KXP = kxp<H>(), HH = H / 2, R1 = S::R1, NJ = H / R1;
+    constexpr int KP = kRows / 2;
+    extern __shared__ float2 sm[];
+    float2* Z = sm;                              // [kRows][PITCH]
+    float2* tw = Z + S::Z;
+    for (int i = threadIdx.x; i < H; i += NT) tw[i] = R.twiddle[i];
+    // first row, flat over (z, y); the V modes take kRows row pairs
+    constexpr bool VV = MODE >= 2;
+    constexpr int PAIR = MODE == 3 ? HH : 1;     // distance of the two rows of a pair
+    constexpr int STEP = MODE == 0 || MODE == 3 ? 1 : 2;   // rows from one complex row to the next
+    constexpr int VB = HH / kRows;               // mode 3: blocks per plane
+    const size_t row0 = MODE == 3 ? static_cast<size_t>(blockIdx.x / VB) * H + (blockIdx.x % VB) * kRows
+                                  : static_cast<size_t>(blockIdx.x) * (MODE == 2 ? 2 * kRows : kRows);
+    const float u_scale = R.sc->u_scale;
+    const float c0 = VV ? *R.voff : 0.0f;   // that spectrum only feeds derivatives
+    const float* v = R.v + row0 * H;
+    const float* m = R.m + row0 * H;
+    const float* w = R.w + row0 * H;
+    unsigned long long* acc = R.acc + row0 * H;
+    const float* us = R.us ? R.us + row0 * H : nullptr;
+    float* vo = R.v_out + row0 * H;
+    constexpr int CH = MODE == 0 ? (R1 % 4 == 0 ? 4 : 2) : 2;
+    static_assert(R1 % CH == 0, "whole chunks");
+    constexpr int NR = MODE == 0 ? 1 : 2;        // real rows per complex row
+#pragma unroll 1
+    for (int b = threadIdx.x; b < kRows * NJ; b += NT) {
+        const int t = b / NJ, j = b % NJ;
+        const int row = STEP * (MODE == 1 ? t % KP : t);
+        const bool want_w = MODE == 0 || (MODE == 1 && t >= KP);   // w* and v^n
+        float2 val[R1];
+#pragma unroll
+        for (int r0 = 0; r0 < R1; r0 += CH) {
+            // all loads of a chunk before its stores
+            float rv[CH][NR], rm[CH][NR], rw[CH][NR], ru[CH][NR];
+            unsigned long long ra[CH][NR];
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+#pragma unroll
+                for (int h = 0; h < NR; ++h) {
+                    const int o = (row + h * PAIR) * H + j + (r0 + c) * NJ;
+                    rv[c][h] = rm[c][h] = rw[c][h] = ru[c][h] = 0.f;
+                    ra[c][h] = 0ull;
+                    if (VV) {
+                        rv[c][h] = vo[o];
+                    } else {
+                        rm[c][h] = m[o];
+                        ra[c][h] = acc[o];
+                        if (us) ru[c][h] = us[o];
+                        if (want_w) {
+                            rv[c][h] = v[o];
+                            rw[c][h] = w[o];
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+                float out[2];
+#pragma unroll
+                for (int h = 0; h < NR; ++h) {
+                    const int o = (row + h * PAIR) * H + j + (r0 + c) * NJ;
+                    const float u = acc_to_float(ra[c][h]) * u_scale;
+                    const float um = us ? ru[c][h] : u;
+                    if (MODE == 0) {
+                        out[0] = react_m(a, rm[c][h], um);
+                        out[1] = react_w(a, rv[c][h], rw[c][h], u);
+                    } else if (MODE == 1) {
+                        out[h] = want_w ? react_w(a, rv[c][h], rw[c][h], u)
+                                        : react_m(a, rm[c][h], um);
+                    } else {
+                        out[h] = rv[c][h] - c0;
+                    }
+                    if (!VV && want_w) vo[o] = react_v(a, rv[c][h], rm[c][h]);
+                }
+                val[r0 + c] = make_float2(out[0], out[1]);
+            }
+        }
+        dft<R1, -1>(val);
+#pragma unroll
+        for (int r = 0; r < R1; ++r) Z[t * S::At::PITCH + j * (R1 + 1) + r] = val[r];
+    }
+    __syncthreads();
+    if (!VV) {
+        ulonglong2* q = reinterpret_cast<ulonglong2*>(acc);
+        for (int i = threadIdx.x; i < kRows * H / 2; i += NT) q[i] = make_ulonglong2(0ull, 0ull);
+    }
+    const typename S::At at{};
+    fft_rest_at<H, V, kRows, NT, -1>(Z, tw, at);
+    for (int q = threadIdx.x; q < kRows * HH; q += NT) {
+        const int t = q / HH, k = q % HH;
+        float2* d1;
+        float2* d2;
+        if (MODE == 0) {
+            d1 = R.specM + (row0 + t) * KXP;
+            d2 = R.specW + (row0 + t) * KXP;
+        } else {
+            d1 = (VV ? R.specV + (row0 + STEP * t) * KXP
+                     : (t < KP ? R.specM : R.specW) + (row0 + STEP * (t % KP)) * KXP);
+            d2 = d1 + PAIR * KXP;
+        }
+        float2 x1, x2;
+        split_modes(Z[at(t, k)], Z[at(t, k == 0 ? 0 : H - k)], x1, x2);
+        d1[k] = x1;
+        d2[k] = x2;
+        if (k == 0) {
+            const float2 zn = Z[at(t, HH)];
+            split_modes(zn, zn, x1, x2);
+            d1[HH] = x1;
+            d2[HH] = x2;
+        }
+    }
+}
+
+// Inverse: two half rows to two real rows per complex transform, kRows
+// transforms per block.  Five neighbouring blocks cover 2 kRows rows: two take
+// (m, w) rows, two (dv/dx, dv/dy) rows, one dv/dz row pairs, so that the components of
+// a node of the gather array are written close together in time, while its
+// line is in L2.  PAIRH: the 2 kRows rows are y0 .. y0 + 7 and the same + H/2,
+// paired across (radix plan 2); else consecutive, paired (2p, 2p + 1).  Half
+// rows feed the first stage in registers and the last stage, its lanes along x,
+// stores to global memory.  (One block for all 20 transforms of 8 rows, storing whole
+// nodes from shared memory, took 234 us at 256^3
+// and 976 us at 384^3, against 169 and 523.)
+template <int H, int V, bool PAIRH>
+__global__ void __launch_bounds__(LineCfg<H>::NTX, row_blocks<H>())
+    k_rows_inverse(const __grid_constant__ SpecBatch<1> batch) {
+    const SpecRun& R = batch.run[0];
+    const SpectralArgs& a = R.a;
+    using S = RowShape<H, V>;
+    using P = Radix<H, V>;
+    constexpr int NT = LineCfg<H>::NTX, KXP = kxp<H>(), HH = H / 2;
+    extern __shared__ float2 sm[];
+    float2* Z = sm;                              // [kRows][PITCH]
+    float2* tw = Z + S::Z;
+    const int group = blockIdx.x / 5, part = blockIdx.x % 5;
+    const int kind = part < 2 ? 0 : part < 4 ? 1 : 2;
+    if (kind == 0 && !a.do_mw) return;           // a state's initial gradient: no m, w
+    for (int i = threadIdx.x; i < H; i += NT) tw[i] = R.twiddle[i];
+    __syncthreads();
+    constexpr int VB = HH / kRows;
+    const size_t g0 = PAIRH ? static_cast<size_t>(group / VB) * H + (group % VB) * kRows
+                            : static_cast<size_t>(group) * (2 * kRows);   // flat over (z, y)
+    const size_t row0 = g0 + (kind == 2 ? 0 : (part & 1) * (PAIRH ? HH : kRows));
+    constexpr int PAIR = PAIRH ? HH : 1;
+    const int step = kind == 2 && !PAIRH ? 2 : 1;        // rows from one transform to the next
+    const float2* s1 = (kind == 0 ? R.specM : kind == 1 ? R.specDx : R.specB) + row0 * KXP;
+    const float2* s2 = kind == 0 ? R.specW + row0 * KXP
+                     : kind == 1 ? R.specDy + row0 * KXP : s1 + PAIR * KXP;
+    const typename S::At at{};
+    auto sload = [=](int t, int p) { return Z[at(t, p)]; };
+    auto sstore = [=](int t, int p, float2 val) { Z[at(t, p)] = val; };
+    stage_ls<H, S::R1, 1, kRows, NT, +1, true, false>(
+        tw,
+        [=](int t, int kx) {
+            const int k = kx <= HH ? kx : H - kx;
+            return pack_modes<H>(s1[t * step * KXP + k], s2[t * step * KXP + k], kx);
+        },
+        sstore);
+    __syncthreads();
+    if constexpr (P::R3 > 1) {
+        stage_ls<H, P::R2, S::R1, kRows, NT, +1, false, true>(tw, sload, sstore);
+        __syncthreads();
+    }
+    if constexpr (P::R4 > 1) {
+        stage_ls<H, P::R3, S::R1 * P::R2, kRows, NT, +1, false, true>(tw, sload, sstore);
+        __syncthreads();
+    }
+    constexpr int RL = P::R4 > 1 ? P::R4 : P::R3 > 1 ? P::R3 : P::R2;
+    const float sc = a.out_scale, sxy = a.out_scale_xy;
+    float* m_out = R.m_out + row0 * H;
+    float* w_out = R.w_out + row0 * H;
+    float* G = R.G + 4 * row0 * H;
+    stage_ls<H, RL, H / RL, kRows, NT, +1, true, false>(
+        tw, sload, [=](int t, int x, float2 val) {
+            const int o = t * step * H + x;
+            if (kind == 0) {
+                const float wv = val.y * sc;
+                m_out[o] = val.x * sc;
+                w_out[o] = wv;
+                G[4 * o + 3] = wv;
+            } else if (kind == 1) {
+                *reinterpret_cast<float2*>(G + 4 * o) = make_float2(val.x * sxy, val.y * sxy);
+            } else {
+                G[4 * o + 2] = val.x * sc;
+                G[4 * (o + PAIR * H) + 2] = val.y * sc;
+            }
+        });
+}
+
+// ---------------------------------------------------------------- launches
+template <class K>
+void allow_smem(K kernel, size_t bytes) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         static_cast<int>(bytes));
+}
+
+// Shared memory of the plane passes.
 template <int H> struct FusedSmem {
     static constexpr size_t fwd = (static_cast<size_t>(H) * rowp<H>() + H * kxp<H>() + H) * sizeof(float2);
-    static constexpr size_t z = (static_cast<size_t>(H) * zcols<H>() + H) * sizeof(float2);
     static constexpr size_t inv = (3 * static_cast<size_t>(H) * kxs<H>() + H) * sizeof(float2);
 };
 
-template <int H, int NB, int V>
-void configure_fused(int device) {
-    static int configured_device = -1;   // attributes are set once per process and device
-    if (configured_device == device) return;
-    cudaFuncSetAttribute(k_forward_xy<H, NB, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(FusedSmem<H>::fwd));
-    cudaFuncSetAttribute(k_z_multiply<H, NB, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(FusedSmem<H>::z));
-    cudaFuncSetAttribute(k_inverse_xy<H, NB, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(FusedSmem<H>::inv));
-    configured_device = device;
-}
-
-// One fused pass over a batch of nb runs of grid size H.
+// One fused pass over a batch of nb runs of grid size H <= 128: 0 forward
+// planes, 1 z lines, 2 inverse planes.
 template <int H, int NB, int V>
 cudaError_t fused_pass(const SpecBatch<NB>& batch, int nb, int pass, int device, cudaStream_t s) {
-    configure_fused<H, NB, V>(device);
-    constexpr int KXP = kxp<H>();
-    if (pass == 0) {
+    static int configured_device = -1;   // attributes are set once per process and device
+    if (configured_device != device) {
+        allow_smem(k_forward_xy<H, NB, V>, FusedSmem<H>::fwd);
+        allow_smem(k_lines_z<H, NB, V>, LineShape<H>::bytes);
+        allow_smem(k_inverse_xy<H, NB, V>, FusedSmem<H>::inv);
+        configured_device = device;
+    }
+    const SpectralArgs& a = batch.run[0].a;   // a batch of several: full steps without the filter
+    if (pass == 0)
         return launch_pdl(k_forward_xy<H, NB, V>, dim3(H, nb), dim3(Cfg<H>::NT1),
                           FusedSmem<H>::fwd, s, batch);
-    } else if (pass == 1) {
-        const int kt = (KXP + zcols<H>() - 1) / zcols<H>();
-        return launch_pdl(k_z_multiply<H, NB, V>, dim3(H, 4, NB == 1 ? kt : nb),
-                          dim3(Cfg<H>::NT2), FusedSmem<H>::z, s, batch);
-    } else {
-        return launch_pdl(k_inverse_xy<H, NB, V>, dim3(2 * H, 1, nb), dim3(Cfg<H>::NT3),
-                          FusedSmem<H>::inv, s, batch);
+    if (pass == 1) {
+        const int f0 = a.do_mw ? 0 : 2, f1 = a.filter ? 4 : 3;
+        return launch_pdl(k_lines_z<H, NB, V>, dim3(LineShape<H>::TC, f1 - f0, nb),
+                          dim3(LineCfg<H>::NT), LineShape<H>::bytes, s, batch, f0);
     }
+    return launch_pdl(k_inverse_xy<H, NB, V>, dim3(2 * H, 1, nb), dim3(Cfg<H>::NT3),
+                      FusedSmem<H>::inv, s, batch);
 }
 
 // One fused pass over n runs (n = 1: the batch-of-one instantiation).
@@ -1092,6 +839,45 @@ cudaError_t fused_runs(const SpecRun* runs, int n, int pass, int device, cudaStr
     SpecBatch<kMaxBatch> batch;
     for (int i = 0; i < n; ++i) batch.run[i] = runs[i];
     return fused_pass<H, kMaxBatch, V>(batch, n, pass, device, s);
+}
+
+// Passes of the per-axis pipeline, grouped like the fused ones: 0 forward
+// (x, y), 1 z, 2 inverse (y, x).  PLAN2: how rows are packed and paired.  Ordinary
+// launches: with programmatic ones the plan kernel on the second stream kept
+// the passes waiting (256^3: 1.49 against 1.31 ms per step).
+template <int H, int V, bool PLAN2>
+cudaError_t axis_pass(const SpecRun& run, int pass, int device, cudaStream_t s) {
+    using L = LineShape<H>;
+    using X = RowShape<H, V>;
+    constexpr int MW = PLAN2 ? 0 : 1, VV = PLAN2 ? 3 : 2;
+    static int configured_device = -1;
+    if (configured_device != device) {
+        allow_smem(k_rows_forward<H, V, MW>, X::bytes);
+        allow_smem(k_rows_forward<H, V, VV>, X::bytes);
+        allow_smem(k_rows_inverse<H, V, PLAN2>, X::bytes);
+        allow_smem(k_lines_y<H, -1, V>, L::bytes);
+        allow_smem(k_lines_y<H, +1, V>, L::bytes);
+        allow_smem(k_lines_z<H, 1, V>, L::bytes);
+        configured_device = device;
+    }
+    SpecBatch<1> one;
+    one.run[0] = run;
+    const SpectralArgs& a = run.a;
+    const dim3 nx(LineCfg<H>::NTX), nl(LineCfg<H>::NT);
+    const unsigned rows = H * H / kRows;
+    const int f0 = a.do_mw ? 0 : 2;
+    if (pass == 0) {
+        if (a.do_mw) k_rows_forward<H, V, MW><<<rows, nx, X::bytes, s>>>(one);
+        k_rows_forward<H, V, VV><<<rows / 2, nx, X::bytes, s>>>(one);
+        k_lines_y<H, -1, V><<<dim3(YTiles<H>::ALL, 3 - f0), nl, L::bytes, s>>>(one, f0);
+    } else if (pass == 1) {
+        const int f1 = a.filter ? 4 : 3;
+        k_lines_z<H, 1, V><<<dim3(L::TC, f1 - f0), nl, L::bytes, s>>>(one, f0);
+    } else {
+        k_lines_y<H, +1, V><<<dim3(YTiles<H>::ALL, 5 - f0), nl, L::bytes, s>>>(one, f0);
+        k_rows_inverse<H, V, PLAN2><<<rows / 2 * 5, nx, X::bytes, s>>>(one);
+    }
+    return cudaGetLastError();
 }
 
 }  // namespace

@@ -347,70 +347,186 @@ __device__ __forceinline__ void fft_axis(float2* buf, const float2* tw) {
     fft_axis_at<L, V, NTRANS, NT, SIGN>(buf, tw, Strided<TS, ES>{});
 }
 
-// A length-L DFT spread over a group of P lanes of one warp (Q = L / P
-// elements per lane, S = Q / P), as the two factors of L = P Q
-// (Cooley-Tukey) with one exchange through the group's shared-memory tile:
-//  * spatial layout: lane l holds n = l + P m in v[m], m < Q;
-//  * spectral layout: lane l holds k = k1 + Q k2 with k1 = S l + s in
-//    v[s P + k2], s < S, k2 < P.
-// to_spectral: DFT_Q over m, twiddle w_L^(l k1), exchange, DFT_P over l.
-// to_spatial reverses it: DFT_P over k2, twiddle w_L^(n1 k1), exchange,
-// DFT_Q over k1.  The tile holds P rows of PITCH float2; __syncwarp orders
-// the exchange, so no block barrier is involved.
-template <int L, int P, int PITCH>
-struct WarpFFT {
-    static constexpr int Q = L / P, S = Q / P;
-    static_assert(Q % P == 0 && PITCH >= Q, "warp FFT shape");
-
-    template <int SIGN>
-    static __device__ __forceinline__ float2 twiddle(const float2* tw, int j) {
-        float2 w = tw[j];
-        if (SIGN > 0) w.y = -w.y;
-        return w;
-    }
-
-    template <int SIGN>
-    static __device__ __forceinline__ void to_spectral(float2 (&v)[Q], int l, float2* ex,
-                                                       const float2* tw) {
-        dft<Q, SIGN>(v);
+// One stage between a loader and a store: element j of transform t is
+// load(t, j), output position p goes to store(t, p, v).  JF: consecutive
+// lanes take consecutive butterflies of one transform (their inputs are
+// neighbours, which is what a load from or a store to global memory wants
+// when transforms lie along rows); otherwise consecutive lanes take
+// consecutive transforms.  INPLACE: the store may overwrite what load reads,
+// so all butterflies are held in registers over a block barrier.  No barrier
+// follows the stores.
+template <int L, int R, int NS, int NTRANS, int NT, int SIGN, bool JF, bool INPLACE, class Load,
+          class Store>
+__device__ __forceinline__ void stage_ls(const float2* tw, Load load, Store store) {
+    constexpr int NJ = L / R, NB = NTRANS * NJ, BPT = (NB + NT - 1) / NT;
+    auto butterfly = [&](int b, float2 (&v)[R]) {
+        const int t = JF ? b / NJ : b % NTRANS, j = JF ? b % NJ : b / NTRANS, k = j % NS;
 #pragma unroll
-        for (int k1 = 1; k1 < Q; ++k1) v[k1] = cmul(v[k1], twiddle<SIGN>(tw, l * k1));
-        __syncwarp();
+        for (int r = 0; r < R; ++r) {
+            float2 x = load(t, j + r * NJ);
+            if (NS > 1 && r > 0) {
+                float2 wv = tw[r * k * (L / (NS * R))];
+                if (SIGN > 0) wv.y = -wv.y;
+                x = cmul(x, wv);
+            }
+            v[r] = x;
+        }
+        dft<R, SIGN>(v);
+    };
+    auto put = [&](int b, const float2 (&v)[R]) {
+        const int t = JF ? b / NJ : b % NTRANS, j = JF ? b % NJ : b / NTRANS, k = j % NS;
 #pragma unroll
-        for (int k1 = 0; k1 < Q; ++k1) ex[l * PITCH + k1] = v[k1];
-        __syncwarp();
+        for (int r = 0; r < R; ++r) store(t, (j - k) * R + k + r * NS, v[r]);
+    };
+    if constexpr (INPLACE) {
+        float2 v[BPT][R];
 #pragma unroll
-        for (int s = 0; s < S; ++s) {
-            float2 u[P];
+        for (int i = 0; i < BPT; ++i) {
+            const int b = threadIdx.x + i * NT;
+            if (b < NB) butterfly(b, v[i]);
+        }
+        __syncthreads();
 #pragma unroll
-            for (int j = 0; j < P; ++j) u[j] = ex[j * PITCH + S * l + s];
-            dft<P, SIGN>(u);
-#pragma unroll
-            for (int k2 = 0; k2 < P; ++k2) v[s * P + k2] = u[k2];
+        for (int i = 0; i < BPT; ++i) {
+            const int b = threadIdx.x + i * NT;
+            if (b < NB) put(b, v[i]);
+        }
+    } else {
+#pragma unroll 1
+        for (int b = threadIdx.x; b < NB; b += NT) {
+            float2 v[R];
+            butterfly(b, v);
+            put(b, v);
         }
     }
+}
 
-    template <int SIGN>
-    static __device__ __forceinline__ void to_spatial(float2 (&v)[Q], int l, float2* ex,
-                                                      const float2* tw) {
-        __syncwarp();
+// The last forward stage, op(t, k, v) on every mode k, and the first stage
+// of the inverse with the radices in reverse order, in registers: the radix-R
+// butterfly that ends the forward transform holds the modes j + r L/R, which
+// are the inputs of the inverse's first radix-R butterfly.  In place; no
+// barrier follows the stores.
+template <int L, int R, int NTRANS, int NT, class Buf, class At, class Op>
+__device__ __forceinline__ void stage_mid(Buf buf, const float2* tw, At at, Op op) {
+    constexpr int NJ = L / R, NB = NTRANS * NJ, BPT = (NB + NT - 1) / NT;
+    float2 v[BPT][R];
 #pragma unroll
-        for (int s = 0; s < S; ++s) {
-            float2 u[P];
+    for (int i = 0; i < BPT; ++i) {
+        const int b = threadIdx.x + i * NT;
+        if (b < NB) {
+            const int t = b % NTRANS, j = b / NTRANS;
 #pragma unroll
-            for (int k2 = 0; k2 < P; ++k2) u[k2] = v[s * P + k2];
-            dft<P, SIGN>(u);
-            const int k1 = S * l + s;
-            ex[k1] = u[0];
+            for (int r = 0; r < R; ++r) {
+                float2 x = buf[at(t, j + r * NJ)];
+                if (r > 0) x = cmul(x, tw[r * j]);
+                v[i][r] = x;
+            }
+            dft<R, -1>(v[i]);
 #pragma unroll
-            for (int j = 1; j < P; ++j) ex[j * PITCH + k1] = cmul(u[j], twiddle<SIGN>(tw, j * k1));
+            for (int r = 0; r < R; ++r) v[i][r] = op(t, j + r * NJ, v[i][r]);
+            dft<R, +1>(v[i]);
         }
-        __syncwarp();
-#pragma unroll
-        for (int k1 = 0; k1 < Q; ++k1) v[k1] = ex[l * PITCH + k1];
-        dft<Q, SIGN>(v);
     }
-};
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < BPT; ++i) {
+        const int b = threadIdx.x + i * NT;
+        if (b < NB) {
+            const int t = b % NTRANS, j = b / NTRANS;
+#pragma unroll
+            for (int r = 0; r < R; ++r) buf[at(t, j * R + r)] = v[i][r];
+        }
+    }
+}
+
+// Whether the plan reads the same backwards (the inverse in reverse order is
+// then the ordinary inverse).
+template <int L, int V> constexpr bool palindromic() {
+    using P = Radix<L, V>;
+    return P::R4 > 1 ? P::R1 == P::R4 && P::R2 == P::R3
+         : P::R3 > 1 ? P::R1 == P::R3 : P::R1 == P::R2;
+}
+
+// Forward DFT, op on every mode, inverse DFT (without 1/L) of NTRANS lines:
+// load(t, j) gives the inputs, store(t, j, v) takes the outputs, buf holds
+// the lines in between, addressed by at.  load may not read buf.  With a
+// palindromic plan the two transforms meet in registers (stage_mid) and a
+// two-radix line crosses shared memory twice, else three times: the inverse
+// takes the radices in the plan's order, so that a mode's rounding does not
+// depend on the kernel that transforms it.  The caller separates the last
+// reads of buf from later writes.
+template <int L, int V, int NTRANS, int NT, class At, class Load, class Op,
+          class Store>
+__device__ __forceinline__ void round_trip(float2* buf, const float2* tw, At at, Load load, Op op,
+                                           Store store) {
+    using P = Radix<L, V>;
+    constexpr int R1 = P::R1, R2 = P::R2, R3 = P::R3, R4 = P::R4;
+    constexpr int RL = R4 > 1 ? R4 : R3 > 1 ? R3 : R2;
+    auto sload = [=](int t, int p) { return buf[at(t, p)]; };
+    auto sstore = [=](int t, int p, float2 v) { buf[at(t, p)] = v; };
+    stage_ls<L, R1, 1, NTRANS, NT, -1, false, false>(tw, load, sstore);
+    __syncthreads();
+    if constexpr (R3 > 1) {
+        stage_ls<L, R2, R1, NTRANS, NT, -1, false, true>(tw, sload, sstore);
+        __syncthreads();
+    }
+    if constexpr (R4 > 1) {
+        stage_ls<L, R3, R1 * R2, NTRANS, NT, -1, false, true>(tw, sload, sstore);
+        __syncthreads();
+    }
+    if constexpr (palindromic<L, V>()) {
+        stage_mid<L, RL, NTRANS, NT>(buf, tw, at, op);
+        __syncthreads();
+        if constexpr (R4 > 1) {
+            stage_ls<L, R3, R4, NTRANS, NT, +1, false, true>(tw, sload, sstore);
+            __syncthreads();
+        }
+        if constexpr (R3 > 1) {
+            stage_ls<L, R2, R3 * R4, NTRANS, NT, +1, false, true>(tw, sload, sstore);
+            __syncthreads();
+        }
+        stage_ls<L, R1, L / R1, NTRANS, NT, +1, false, false>(tw, sload, store);
+    } else {
+        stage_ls<L, RL, L / RL, NTRANS, NT, -1, false, true>(
+            tw, sload, [=](int t, int k, float2 v) { buf[at(t, k)] = op(t, k, v); });
+        __syncthreads();
+        stage_ls<L, R1, 1, NTRANS, NT, +1, false, true>(tw, sload, sstore);
+        __syncthreads();
+        if constexpr (R3 > 1) {
+            stage_ls<L, R2, R1, NTRANS, NT, +1, false, true>(tw, sload, sstore);
+            __syncthreads();
+        }
+        if constexpr (R4 > 1) {
+            stage_ls<L, R3, R1 * R2, NTRANS, NT, +1, false, true>(tw, sload, sstore);
+            __syncthreads();
+        }
+        stage_ls<L, RL, L / RL, NTRANS, NT, +1, false, false>(tw, sload, store);
+    }
+}
+
+// One DFT of NTRANS lines from load to store through buf; JF1 and JFL: the
+// lane order of the first and of the last stage (see stage_ls).
+template <int L, int V, int NTRANS, int NT, int SIGN, bool JF1, bool JFL, class At, class Load,
+          class Store>
+__device__ __forceinline__ void one_way(float2* buf, const float2* tw, At at, Load load,
+                                        Store store) {
+    using P = Radix<L, V>;
+    constexpr int R1 = P::R1, R2 = P::R2, R3 = P::R3, R4 = P::R4;
+    constexpr int RL = R4 > 1 ? R4 : R3 > 1 ? R3 : R2;
+    auto sload = [=](int t, int p) { return buf[at(t, p)]; };
+    auto sstore = [=](int t, int p, float2 v) { buf[at(t, p)] = v; };
+    stage_ls<L, R1, 1, NTRANS, NT, SIGN, JF1, false>(tw, load, sstore);
+    __syncthreads();
+    if constexpr (R3 > 1) {
+        stage_ls<L, R2, R1, NTRANS, NT, SIGN, false, true>(tw, sload, sstore);
+        __syncthreads();
+    }
+    if constexpr (R4 > 1) {
+        stage_ls<L, R3, R1 * R2, NTRANS, NT, SIGN, false, true>(tw, sload, sstore);
+        __syncthreads();
+    }
+    stage_ls<L, RL, L / RL, NTRANS, NT, SIGN, JFL, false>(tw, sload, store);
+}
 
 }  // namespace fftk
 }  // namespace sipf

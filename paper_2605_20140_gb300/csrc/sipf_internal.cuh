@@ -166,7 +166,7 @@ struct SpectralArgs {
     int do_mw;             // transform m and w (0 in the initial transform)
 };
 
-// One run's data for the fused spectral passes (H <= 128).  The passes take
+// One run's data for the spectral passes.  The fused passes (H <= 128) take
 // a batch of runs as a launch parameter: one run for a context's own step,
 // up to kMaxBatch runs of one grid size for an ensemble's batched step (the
 // run is then a grid dimension of the launch).
@@ -186,7 +186,7 @@ struct SpecRun {
     float2* specB;
     float2* specA;                // filtered v spectrum (filter on only)
     float2* specDx;               // i k_x V and i k_y V after the inverse y pass
-    float2* specDy;               // (per-axis pipelines only)
+    float2* specDy;               // (per-axis pipeline only)
     const float2* twiddle;
     float* voff;
     const StepScalars* sc;        // scalars of the step (u_bar per accumulator unit)
@@ -284,7 +284,7 @@ struct sipf_ctx {
     float2* specV = nullptr;
     float2* specB = nullptr;
     float2* specA = nullptr;         // filtered v spectrum (filter on only)
-    float2* specDx = nullptr;        // i k_x V, i k_y V after the inverse y pass (H > 128 only)
+    float2* specDx = nullptr;        // i k_x V, i k_y V after the inverse y pass (per-axis only)
     float2* specDy = nullptr;
     float2* twiddle = nullptr;       // exp(-2 pi i j / H), j < H
     float* voff = nullptr;           // device scalar: offset subtracted from v before its FFT
@@ -376,7 +376,7 @@ int resample_device(sipf_ctx* c, int src, int dst, double ratio, int* done, std:
 cudaError_t launch_spectral_step(sipf_ctx* c, const SpectralArgs& a);
 cudaError_t launch_spectral_pass(sipf_ctx* c, const SpectralArgs& a, int pass);
 // The context's data for the fused spectral passes (its current buffer parity).
-bool has_warp_pipeline(int H);
+bool has_axis_pipeline(int H);   // radix plan 2: the per-axis passes
 SpecRun spec_run(const sipf_ctx* c, const SpectralArgs& a);
 // One fused spectral pass (0 forward, 1 z, 2 inverse) over n <= kMaxBatch
 // runs of grid size H <= 128, in one launch.
