@@ -22,6 +22,7 @@
 // tile reserve consecutive slots with one global atomic.  A one-block plan
 // kernel then builds the next step's items and the next bucket layout from
 // the counts.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -728,7 +729,8 @@ __global__ void __launch_bounds__(kNT, DepBlock<ORDER>::MIN_BLOCKS)
 
 // ------------------------------------------------------------------ planning
 // Block-wide exclusive scan (one value per thread) of kPlanNT threads.
-constexpr int kPlanNT = 1024;
+constexpr int kPlanNT = 512;
+constexpr int kPlanCluster = 8;   // blocks of the plan kernel on large grids
 
 __device__ __forceinline__ int block_exclusive_scan(int v, int* smem, int* total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -758,6 +760,25 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* smem, int* total
     return r;
 }
 
+// Exclusive scan of three ints per lane over a warp; the totals in every lane.
+__device__ __forceinline__ int3 warp_exclusive_scan3(int3 v, int3* total) {
+    const int lane = threadIdx.x & 31;
+    int3 s = v;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int x = __shfl_up_sync(kFull, s.x, off), y = __shfl_up_sync(kFull, s.y, off);
+        const int z = __shfl_up_sync(kFull, s.z, off);
+        if (lane >= off) {
+            s.x += x;
+            s.y += y;
+            s.z += z;
+        }
+    }
+    *total = make_int3(__shfl_sync(kFull, s.x, 31), __shfl_sync(kFull, s.y, 31),
+                       __shfl_sync(kFull, s.z, 31));
+    return make_int3(s.x - v.x, s.y - v.y, s.z - v.z);
+}
+
 // From the counts of buffer `b` (just written): the items that read it next
 // (tile buckets split into kItem chunks, then the overflow region) with
 // their offsets in the compacted particle order; and, when next_cnt is not
@@ -765,7 +786,13 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* smem, int* total
 // count + count/slack_div + slack_add, rounded up to a multiple of 4; the
 // context's buffers hold at least slack_div = 8, slack_add = 32) with its
 // counters reset; with next_sc, the next step's scalars from those of this
-// step.
+// step.  Run by CL blocks (a cluster): each warp takes consecutive strips of 32
+// tiles, sums them, gets its offsets from a scan over the warps and (through
+// distributed shared memory) over the blocks, then reads its strips again
+// and writes, a warp together for a tile of many items.  Bound by the latency
+// of the chain, so by the strips per warp: 282 us as one block of 1024 threads
+// with a tile per thread and step (256^3 / 2^25, ncu), 46 us as this cluster.
+template <int CL>
 __device__ __forceinline__ void plan_body(
     int ntiles, int T, const int* __restrict__ cnt, const int* __restrict__ cap,
     const int* __restrict__ bstart, const int* __restrict__ ovf, int ovf_base, Item* items,
@@ -773,64 +800,118 @@ __device__ __forceinline__ void plan_body(
     int* __restrict__ status, const StepScalars* __restrict__ cur_sc,
     StepScalars* __restrict__ next_sc, double dt, double log2_maxrel, double exp_logref,
     double h3, int slack_div, int slack_add) {
-    __shared__ int smem[33];
-    const int per = (ntiles + kPlanNT - 1) / kPlanNT;
-    const int t0 = threadIdx.x * per;
-    int my_items = 0, my_fill = 0, my_cap = 0;
-    for (int k = 0; k < per; ++k) {
-        const int t = t0 + k;
-        if (t >= ntiles) break;
-        const int c = cnt[t];
-        const int f = min(c, cap[t]);
-        my_items += (f + kItem - 1) / kItem;
-        my_fill += f;
-        if (next_cnt) my_cap += ((c + c / slack_div + slack_add) + 3) & ~3;
+    constexpr int NW = kPlanNT / 32;
+    constexpr int kOwnItems = 4;
+    __shared__ int3 warp_base[NW];
+    __shared__ int3 block_total;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int rank = 0;
+    if constexpr (CL > 1) rank = static_cast<int>(cooperative_groups::this_cluster().block_rank());
+    const int strips = (ntiles + 31) / 32, per = (strips + CL * NW - 1) / (CL * NW);
+    const int s0 = min((rank * NW + warp) * per, strips), s1 = min(s0 + per, strips);
+    // items, particles in the bucket and next capacity of this lane's tile of strip s
+    auto counts = [&](int s, int& c) {
+        const int t = s * 32 + lane;
+        int3 v = make_int3(0, 0, 0);
+        c = 0;
+        if (t < ntiles) {
+            c = cnt[t];
+            v.y = min(c, cap[t]);
+            v.x = (v.y + kItem - 1) / kItem;
+            if (next_cnt) v.z = ((c + c / slack_div + slack_add) + 3) & ~3;
+        }
+        return v;
+    };
+    int c;
+    int3 sum = make_int3(0, 0, 0), tot;
+    for (int s = s0; s < s1; ++s) {
+        const int3 v = counts(s, c);
+        sum.x += v.x;
+        sum.y += v.y;
+        sum.z += v.z;
     }
-    int tot_items, tot_fill, tot_cap;
-    int item0 = block_exclusive_scan(my_items, smem, &tot_items);
-    int out0 = block_exclusive_scan(my_fill, smem, &tot_fill);
-    int cap0 = next_cnt ? block_exclusive_scan(my_cap, smem, &tot_cap) : 0;
-    for (int k = 0; k < per; ++k) {
-        const int t = t0 + k;
-        if (t >= ntiles) break;
-        const int c = cnt[t];
-        const int f = min(c, cap[t]);
-        for (int q = 0; q * kItem < f; ++q) {
-            Item it;
-            it.tile = t;
-            it.beg = bstart[t] + q * kItem;
-            it.end = bstart[t] + min((q + 1) * kItem, f);
-            it.out = out0 + q * kItem;
-            it.tx = t % T;
-            it.ty = (t / T) % T;
-            it.tz = t / (T * T);
-            it.pad = 0;
-            items[item0++] = it;
+    warp_exclusive_scan3(sum, &tot);
+    if (lane == 0) warp_base[warp] = tot;
+    __syncthreads();
+    if (warp == 0) {
+        const int3 v = lane < NW ? warp_base[lane] : make_int3(0, 0, 0);
+        const int3 ex = warp_exclusive_scan3(v, &tot);
+        if (lane < NW) warp_base[lane] = ex;
+        if (lane == 0) block_total = tot;
+    }
+    __syncthreads();
+    int3 off = warp_base[warp], all = block_total;
+    if constexpr (CL > 1) {
+        namespace cg = cooperative_groups;
+        cg::cluster_group cluster = cg::this_cluster();
+        cluster.sync();
+        all = make_int3(0, 0, 0);
+#pragma unroll
+        for (int r = 0; r < CL; ++r) {
+            const int3 o = *cluster.map_shared_rank(&block_total, r);
+            if (r < rank) {
+                off.x += o.x;
+                off.y += o.y;
+                off.z += o.z;
+            }
+            all.x += o.x;
+            all.y += o.y;
+            all.z += o.z;
         }
-        out0 += f;
-        if (next_cnt) {
-            const int cp = ((c + c / slack_div + slack_add) + 3) & ~3;
-            next_bstart[t] = cap0;
-            next_cap[t] = cp;
+        cluster.sync();   // every block has read the totals
+    }
+    for (int s = s0; s < s1; ++s) {
+        const int3 v = counts(s, c);
+        const int3 ex = warp_exclusive_scan3(v, &tot);
+        const int t = s * 32 + lane;
+        if (next_cnt && t < ntiles) {
+            next_bstart[t] = off.z + ex.z;
+            next_cap[t] = v.z;
             next_cnt[t] = 0;
-            cap0 += cp;
         }
+        const int beg = t < ntiles ? bstart[t] : 0;
+        auto put = [&](int tile, int q, int b0, int fill, int item0, int out0) {
+            Item it;
+            it.tile = tile;
+            it.beg = b0 + q * kItem;
+            it.end = b0 + min((q + 1) * kItem, fill);
+            it.out = out0 + q * kItem;
+            it.tx = tile % T;
+            it.ty = (tile / T) % T;
+            it.tz = tile / (T * T);
+            it.pad = 0;
+            items[item0 + q] = it;
+        };
+        // the first items of every tile at once, a lane per tile; what a tile has
+        // beyond them by the whole warp, tile by tile
+        for (int q = 0; q < min(v.x, kOwnItems); ++q)
+            put(t, q, beg, v.y, off.x + ex.x, off.y + ex.y);
+        for (unsigned left = __ballot_sync(kFull, v.x > kOwnItems); left; left &= left - 1) {
+            const int o = __ffs(left) - 1;
+            const int n = __shfl_sync(kFull, v.x, o), f = __shfl_sync(kFull, v.y, o);
+            const int b0 = __shfl_sync(kFull, beg, o), i0 = off.x + __shfl_sync(kFull, ex.x, o);
+            const int o0 = off.y + __shfl_sync(kFull, ex.y, o);
+            for (int q = kOwnItems + lane; q < n; q += 32) put(s * 32 + o, q, b0, f, i0, o0);
+        }
+        off.x += tot.x;
+        off.y += tot.y;
+        off.z += tot.z;
+    }
+    if (rank != 0) return;
+    const int no = *ovf;
+    for (int q = threadIdx.x; q < (no + kItem - 1) / kItem; q += kPlanNT) {
+        Item it;
+        it.tile = -1;
+        it.beg = ovf_base + q * kItem;
+        it.end = ovf_base + min((q + 1) * kItem, no);
+        it.out = all.y + q * kItem;
+        it.tx = it.ty = it.tz = it.pad = 0;
+        items[all.x + q] = it;
     }
     if (threadIdx.x == 0) {
-        const int no = *ovf;
-        int n = tot_items;
-        for (int q = 0; q * kItem < no; ++q) {
-            Item it;
-            it.tile = -1;
-            it.beg = ovf_base + q * kItem;
-            it.end = ovf_base + min((q + 1) * kItem, no);
-            it.out = tot_fill + q * kItem;
-            it.tx = it.ty = it.tz = it.pad = 0;
-            items[n++] = it;
-        }
-        *n_items = n;
+        *n_items = all.x + (no + kItem - 1) / kItem;
         if (next_ovf) *next_ovf = 0;
-        if (tot_fill + no < 0) atomicOr(status, kStatusTotal);
+        if (all.y + no < 0) atomicOr(status, kStatusTotal);
         // scalars of the next step: n + 1 at time t_n = t_{n-1} + dt
         if (next_sc)
             fill_step_scalars(next_sc, cur_sc->n + 1u, cur_sc->time + dt, log2_maxrel, exp_logref,
@@ -838,6 +919,7 @@ __device__ __forceinline__ void plan_body(
     }
 }
 
+template <int CL>
 __global__ void __launch_bounds__(kPlanNT)
     k_plan(int ntiles, int T, const int* __restrict__ cnt, const int* __restrict__ cap,
            const int* __restrict__ bstart, const int* __restrict__ ovf, int ovf_base, Item* items,
@@ -845,9 +927,9 @@ __global__ void __launch_bounds__(kPlanNT)
            int* __restrict__ status, const StepScalars* __restrict__ cur_sc,
            StepScalars* __restrict__ next_sc, double dt, double log2_maxrel, double exp_logref,
            double h3, int slack_div, int slack_add) {
-    plan_body(ntiles, T, cnt, cap, bstart, ovf, ovf_base, items, n_items, next_bstart, next_cap,
-              next_cnt, next_ovf, status, cur_sc, next_sc, dt, log2_maxrel, exp_logref, h3,
-              slack_div, slack_add);
+    plan_body<CL>(ntiles, T, cnt, cap, bstart, ovf, ovf_base, items, n_items, next_bstart, next_cap,
+                  next_cnt, next_ovf, status, cur_sc, next_sc, dt, log2_maxrel, exp_logref, h3,
+                  slack_div, slack_add);
 }
 
 // The plan of every run of an ensemble after a batched step from buffer
@@ -857,7 +939,7 @@ __global__ void __launch_bounds__(kPlanNT) k_plan_multi(const RunDesc* __restric
                                                         int parity) {
     const RunDesc& d = runs[blockIdx.x];
     const int b = parity ^ 1, o = parity;
-    plan_body(d.ntiles, d.H / 8, d.cnt[b], d.cap[b], d.bstart[b], d.ovf[b], d.ovf_base, d.items,
+    plan_body<1>(d.ntiles, d.H / 8, d.cnt[b], d.cap[b], d.bstart[b], d.ovf[b], d.ovf_base, d.items,
               d.n_items, d.bstart[o], d.cap[o], d.cnt[o], d.ovf[o], d.status, d.dsc + o,
               d.dsc + b, d.dt, d.log2_maxrel, d.exp_logref, d.h3, d.slack_div, d.slack_add);
 }
@@ -1313,18 +1395,32 @@ cudaError_t launch_step_kernel(sipf_ctx* c, const PushArgs& a, int do_deposit, i
                       c->status);
 }
 
-// Items of buffer `b` and, with next_layout, the layout of b ^ 1.
+// Items of buffer `b` and, with next_layout, the layout of b ^ 1.  One block of
+// 32 warps up to 1024 tiles (H = 80), a strip or less per warp; a cluster of
+// eight beyond.
 cudaError_t launch_plan(sipf_ctx* c, int b, int next_layout, cudaStream_t s, double dt) {
     const int o = b ^ 1;
-    k_plan<<<1, kPlanNT, 0, s>>>(
-        c->ntiles, c->H / 8, c->cnt[b], c->cap[b], c->bstart[b], c->ovf[b], c->ovf_base, c->items,
-        c->n_items, next_layout ? c->bstart[o] : nullptr,
+    const bool cluster = c->ntiles > 2 * kPlanNT;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cluster ? kPlanCluster : 1);
+    cfg.blockDim = dim3(kPlanNT);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kPlanCluster;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster ? 1 : 0;
+    return cudaLaunchKernelEx(
+        &cfg, cluster ? k_plan<kPlanCluster> : k_plan<1>, c->ntiles, c->H / 8,
+        static_cast<const int*>(c->cnt[b]), static_cast<const int*>(c->cap[b]),
+        static_cast<const int*>(c->bstart[b]), static_cast<const int*>(c->ovf[b]), c->ovf_base,
+        c->items, c->n_items, next_layout ? c->bstart[o] : nullptr,
         next_layout ? c->cap[o] : nullptr, next_layout ? c->cnt[o] : nullptr,
         next_layout ? c->ovf[o] : nullptr, c->status,
         // b is the buffer the step just wrote: its slot is the next step's, o's the current one
-        c->dsc + o, dt > 0.0 ? c->dsc + b : nullptr, dt, c->log2_maxrel, c->exp_logref, c->h3,
-        c->slack_div, c->slack_add);
-    return cudaGetLastError();
+        static_cast<const StepScalars*>(c->dsc + o), dt > 0.0 ? c->dsc + b : nullptr, dt,
+        c->log2_maxrel, c->exp_logref, c->h3, c->slack_div, c->slack_add);
 }
 
 cudaError_t launch_step_multi(const RunDesc* runs, int n, int parity, cudaStream_t s) {
