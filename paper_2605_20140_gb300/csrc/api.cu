@@ -192,7 +192,7 @@ size_t ctx_device_bytes(int H, int64_t N, bool filter, bool smoothing) {
     const size_t S = static_cast<size_t>(z.buf_slots);
     size_t b = 2 * (S * (3 * sizeof(float) + sizeof(double) + sizeof(uint32_t)) +
                     3 * static_cast<size_t>(z.ntiles) * sizeof(int) + sizeof(int));
-    b += static_cast<size_t>(z.max_items) * sizeof(Item) + 2 * sizeof(int);
+    b += static_cast<size_t>(z.max_items) * sizeof(Item) + 3 * sizeof(int);
     b += z.H3 * sizeof(int32_t) + (z.H3 + 1) * sizeof(int32_t) +
          (static_cast<size_t>(scan_tiles(static_cast<int>(z.H3))) + 1) * sizeof(int32_t);
     b += z.H3 * sizeof(long long) + 3 * z.H3 * sizeof(float) + 4 * z.H3 * sizeof(float);
@@ -615,7 +615,7 @@ int create_in_pool(const sipf_grid* grid, int64_t N, const sipf_params* params,
              da(&c->cnt[b], c->ntiles) == cudaSuccess && da(&c->ovf[b], 1) == cudaSuccess;
     }
     ok = ok && da(&c->items, static_cast<size_t>(c->max_items)) == cudaSuccess &&
-         da(&c->n_items, 1) == cudaSuccess && da(&c->work, 1) == cudaSuccess &&
+         da(&c->n_items, 2) == cudaSuccess && da(&c->work, 1) == cudaSuccess &&
          da(&c->count, H3) == cudaSuccess && da(&c->cell_start, H3 + 1) == cudaSuccess &&
          da(&c->scan_tmp, static_cast<size_t>(scan_tiles(static_cast<int>(H3))) + 1) == cudaSuccess &&
          da(&c->acc, H3) == cudaSuccess && da(&c->v, H3) == cudaSuccess &&

@@ -297,8 +297,19 @@ struct Layout {
 constexpr int kNT = 256;                  // threads of the step kernel
 constexpr int kPT = 4;                    // particles per thread and item
 constexpr int kItem = kNT * kPT;          // particles per item
+
+// Forms of the step kernel.  Dense: blocks take equal numbers of items, and all
+// kPT chunks (kNT particles) of an item in a loop of fixed length.  Sparse (few
+// particles per tile): a warp takes only the chunks that hold an element for it.
+// Split (few items, in tiles of several chunks): as sparse, but the shares are
+// cut between chunks, in work units: kUnit per chunk and kUnitTile for entering a
+// tile (its gather block read, its node sums written out), so that more blocks
+// have work.  Shares by units do not pay for dense runs (128^3 / 2^22: 110 against
+// 108 us; with kUnitTile = 0 143, since blocks with many thin tiles run long).
+enum Form { kDense, kSparse, kSplit };
+constexpr int kUnit = 2, kUnitTile = 2;
 constexpr int kBlock = 9 * 9 * 9;         // nodes of a tile's gather block
-constexpr int kSparsePerTile = 256;       // below this mean tile occupancy, skip idle warps
+constexpr int kSparsePerTile = 256;       // below this mean tile occupancy: sparse form
 
 // Deposit node block of a tile for assignment order ORDER: local node
 // coordinates [-DO, 8 + DO] per axis (trilinear: the cells' corners 0..8;
@@ -382,6 +393,7 @@ struct StepView {
     Buf src, dst;
     Layout L;
     const Item* items;
+    int n_items;
     unsigned long long* acc;
     int* status;
     int do_deposit, do_move;
@@ -409,12 +421,28 @@ template <int ORDER> struct StepShared {
     int tslot[2];                         // capacity and first slot of the item tile's bucket
 };
 
-// Items [i_lo, i_hi) of one run: deposit of X^(n-1), gather, noise, push,
-// mass update and binning of every particle.  dep and dep64 are zero on entry
-// and on exit.
-template <int ORDER, bool SKIP, class Keys>
-__device__ __forceinline__ void step_items(const StepView& v, const Keys& keys, int i_lo, int i_hi,
+// The last of n_items items whose first work unit is at most u (item 0 if none
+// is): a 32-way search by every warp.
+__device__ __forceinline__ int find_item(const Item* items, int n_items, int u) {
+    const int lane = threadIdx.x & 31;
+    int a = 0, n = n_items;
+    while (n > 1) {
+        const int w = (n + 31) / 32, o = lane * w;
+        const unsigned m = __ballot_sync(kFull, o < n && __ldg(&items[a + o].unit0) <= u);
+        const int k = m ? 31 - __clz(m) : 0;
+        a += k * w;
+        n = min(w, n - k * w);
+    }
+    return a;
+}
+
+// A share of one run: items [u_lo, u_hi), or (split form) the chunks whose first
+// work unit lies in [u_lo, u_hi): deposit of X^(n-1), gather, noise, push, mass update and
+// binning of every particle.  dep and dep64 are zero on entry and on exit.
+template <int ORDER, int FORM, class Keys>
+__device__ __forceinline__ void step_items(const StepView& v, const Keys& keys, int u_lo, int u_hi,
                                            StepShared<ORDER>& sh) {
+    if (u_lo >= u_hi) return;
     using DB = DepBlock<ORDER>;
     // Item sums in 32 bits: the trilinear contributions are non-negative and
     // below 2^19.5 (the deposit scale's bound), so kFlushItems items (4096
@@ -443,10 +471,22 @@ __device__ __forceinline__ void step_items(const StepView& v, const Keys& keys, 
     const int do_deposit = v.do_deposit, do_move = v.do_move;
     int cur = -1, cx0 = 0, cy0 = 0, cz0 = 0;   // tile held in dep64 / gblk, its first cell
     int pending = 0;                           // items summed in dep since its last flush
-    for (int item_idx = i_lo; item_idx <= i_hi; ++item_idx) {
-        const Item it = item_idx < i_hi ? v.items[item_idx] : Item{-1, 0, 0, 0, 0, 0, 0, 0};
-        const int tile = it.tile;
-        if (threadIdx.x < 5 && item_idx + 1 < i_hi) {
+    int item_idx = FORM == kSplit ? find_item(v.items, v.n_items, u_lo) : u_lo;
+    for (;; ++item_idx) {
+        Item it{-1, 0, 0, 0, 0, 0, 0, u_hi};
+        if (FORM == kSplit ? item_idx < v.n_items : item_idx < u_hi) it = v.items[item_idx];
+        // split: chunks j_lo .. j_hi - 1 of this item are this block's
+        int j_lo = 0, j_hi = kPT;
+        bool last = item_idx >= u_hi;
+        if constexpr (FORM == kSplit) {
+            const int n_chunk = (it.end - it.beg + kNT - 1) / kNT;
+            j_lo = max(0, (u_lo - it.unit0 + kUnit - 1) / kUnit);
+            j_hi = min(n_chunk, (u_hi - it.unit0 + kUnit - 1) / kUnit);
+            last = it.unit0 >= u_hi;
+            if (!last && j_lo >= j_hi) continue;    // the first item found may end before u_lo
+        }
+        const int tile = last ? -1 : it.tile;
+        if (threadIdx.x < 5 && !last && item_idx + 1 < (FORM == kSplit ? v.n_items : u_hi)) {
             // the next item's particles are read in about one item's time: have
             // them in L2 by then (one array per thread)
             const Item nx = v.items[item_idx + 1];
@@ -490,7 +530,7 @@ __device__ __forceinline__ void step_items(const StepView& v, const Keys& keys, 
                     }
                 }
             }
-            if (item_idx == i_hi) break;
+            if (last) break;
             cur = tile;
             cx0 = it.tx * 8;
             cy0 = it.ty * 8;
@@ -516,16 +556,16 @@ __device__ __forceinline__ void step_items(const StepView& v, const Keys& keys, 
         }
         __syncthreads();
         int bad = 0;
-        // SKIP: only the iterations with an element for this warp (short items,
-        // common in small runs, leave whole warps idle; the count is
-        // warp-uniform, so the warp-wide votes below see whole warps).  Dense
-        // runs take all kPT iterations, which keeps a register free.
-        int jn = kPT;
-        if constexpr (SKIP) {
+        // sparse and split: only the chunks with an element for this warp
+        // (short items leave whole warps idle; the count is warp-uniform, so the
+        // warp-wide votes below see whole warps).  Dense runs do without the test,
+        // which keeps a register free.
+        int jn = j_hi;
+        if constexpr (FORM != kDense) {
             const int wfirst = it.beg + static_cast<int>(threadIdx.x & ~31u);
-            jn = it.end > wfirst ? min(kPT, (it.end - wfirst + kNT - 1) / kNT) : 0;
+            jn = it.end > wfirst ? min(j_hi, (it.end - wfirst + kNT - 1) / kNT) : 0;
         }
-        for (int j = 0; j < jn; ++j) {
+        for (int j = j_lo; j < jn; ++j) {
             const int e = j * kNT + threadIdx.x;     // element of the item, coalesced
             const int i = it.beg + e;
             const bool valid = i < it.end;
@@ -703,7 +743,7 @@ __device__ __forceinline__ void step_items(const StepView& v, const Keys& keys, 
     }
 }
 
-template <int ORDER, bool SKIP>
+template <int ORDER, int FORM>
 __global__ void __launch_bounds__(kNT, DepBlock<ORDER>::MIN_BLOCKS)
     k_step(PushArgs a, const StepScalars* __restrict__ sc, const float4* __restrict__ G, Buf src,
            Buf dst, Layout L, const Item* __restrict__ items, const int* __restrict__ n_items,
@@ -716,15 +756,15 @@ __global__ void __launch_bounds__(kNT, DepBlock<ORDER>::MIN_BLOCKS)
         sh.dep64[i] = 0;
     }
     pdl_wait();   // the gather array of the spectral passes before
-    // block b takes a contiguous run of items; consecutive items of one tile
-    // share the node block of the gather array and the deposit sums, which
-    // go to the grid accumulator once, when the tile changes
-    const int total = *n_items;
-    const int i_lo = static_cast<int>(static_cast<long long>(blockIdx.x) * total / gridDim.x);
-    const int i_hi = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * total / gridDim.x);
+    // block b takes a contiguous run of items (or work units); consecutive items of
+    // one tile share the node block of the gather array and the deposit sums,
+    // which go to the grid accumulator once, when the tile changes
+    const int total = FORM == kSplit ? n_items[1] : n_items[0];
+    const int u_lo = static_cast<int>(static_cast<long long>(blockIdx.x) * total / gridDim.x);
+    const int u_hi = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * total / gridDim.x);
     const StepView v{a.H, a.drift, a.noise, a.tau, a.k0, a.k1, a.push, sc, G, src, dst, L,
-                     items, acc, status, do_deposit, do_move};
-    step_items<ORDER, SKIP>(v, KeysGiven{a.rk}, i_lo, i_hi, sh);
+                     items, n_items[0], acc, status, do_deposit, do_move};
+    step_items<ORDER, FORM>(v, KeysGiven{a.rk}, u_lo, u_hi, sh);
 }
 
 // ------------------------------------------------------------------ planning
@@ -760,28 +800,29 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* smem, int* total
     return r;
 }
 
-// Exclusive scan of three ints per lane over a warp; the totals in every lane.
-__device__ __forceinline__ int3 warp_exclusive_scan3(int3 v, int3* total) {
+// Exclusive scan of four ints per lane over a warp; the totals in every lane.
+__device__ __forceinline__ int4 warp_exclusive_scan4(int4 v, int4* total) {
     const int lane = threadIdx.x & 31;
-    int3 s = v;
+    int4 s = v;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
         const int x = __shfl_up_sync(kFull, s.x, off), y = __shfl_up_sync(kFull, s.y, off);
-        const int z = __shfl_up_sync(kFull, s.z, off);
+        const int z = __shfl_up_sync(kFull, s.z, off), w = __shfl_up_sync(kFull, s.w, off);
         if (lane >= off) {
             s.x += x;
             s.y += y;
             s.z += z;
+            s.w += w;
         }
     }
-    *total = make_int3(__shfl_sync(kFull, s.x, 31), __shfl_sync(kFull, s.y, 31),
-                       __shfl_sync(kFull, s.z, 31));
-    return make_int3(s.x - v.x, s.y - v.y, s.z - v.z);
+    *total = make_int4(__shfl_sync(kFull, s.x, 31), __shfl_sync(kFull, s.y, 31),
+                       __shfl_sync(kFull, s.z, 31), __shfl_sync(kFull, s.w, 31));
+    return make_int4(s.x - v.x, s.y - v.y, s.z - v.z, s.w - v.w);
 }
 
 // From the counts of buffer `b` (just written): the items that read it next
 // (tile buckets split into kItem chunks, then the overflow region) with
-// their offsets in the compacted particle order; and, when next_cnt is not
+// their offsets in the compacted particle order and in chunks; and, when next_cnt is not
 // null, the bucket layout of the other buffer for the next step (capacity
 // count + count/slack_div + slack_add, rounded up to a multiple of 4; the
 // context's buffers hold at least slack_div = 8, slack_add = 32) with its
@@ -802,67 +843,72 @@ __device__ __forceinline__ void plan_body(
     double h3, int slack_div, int slack_add) {
     constexpr int NW = kPlanNT / 32;
     constexpr int kOwnItems = 4;
-    __shared__ int3 warp_base[NW];
-    __shared__ int3 block_total;
+    __shared__ int4 warp_base[NW];
+    __shared__ int4 block_total;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int rank = 0;
     if constexpr (CL > 1) rank = static_cast<int>(cooperative_groups::this_cluster().block_rank());
     const int strips = (ntiles + 31) / 32, per = (strips + CL * NW - 1) / (CL * NW);
     const int s0 = min((rank * NW + warp) * per, strips), s1 = min(s0 + per, strips);
-    // items, particles in the bucket and next capacity of this lane's tile of strip s
+    // items, particles in the bucket, next capacity and chunks of this lane's
+    // tile of strip s
     auto counts = [&](int s, int& c) {
         const int t = s * 32 + lane;
-        int3 v = make_int3(0, 0, 0);
+        int4 v = make_int4(0, 0, 0, 0);
         c = 0;
         if (t < ntiles) {
             c = cnt[t];
             v.y = min(c, cap[t]);
             v.x = (v.y + kItem - 1) / kItem;
+            v.w = v.y ? kUnitTile + kUnit * ((v.y + kNT - 1) / kNT) : 0;
             if (next_cnt) v.z = ((c + c / slack_div + slack_add) + 3) & ~3;
         }
         return v;
     };
     int c;
-    int3 sum = make_int3(0, 0, 0), tot;
+    int4 sum = make_int4(0, 0, 0, 0), tot;
     for (int s = s0; s < s1; ++s) {
-        const int3 v = counts(s, c);
+        const int4 v = counts(s, c);
         sum.x += v.x;
         sum.y += v.y;
         sum.z += v.z;
+        sum.w += v.w;
     }
-    warp_exclusive_scan3(sum, &tot);
+    warp_exclusive_scan4(sum, &tot);
     if (lane == 0) warp_base[warp] = tot;
     __syncthreads();
     if (warp == 0) {
-        const int3 v = lane < NW ? warp_base[lane] : make_int3(0, 0, 0);
-        const int3 ex = warp_exclusive_scan3(v, &tot);
+        const int4 v = lane < NW ? warp_base[lane] : make_int4(0, 0, 0, 0);
+        const int4 ex = warp_exclusive_scan4(v, &tot);
         if (lane < NW) warp_base[lane] = ex;
         if (lane == 0) block_total = tot;
     }
     __syncthreads();
-    int3 off = warp_base[warp], all = block_total;
+    int4 off = warp_base[warp], all = block_total;
     if constexpr (CL > 1) {
         namespace cg = cooperative_groups;
         cg::cluster_group cluster = cg::this_cluster();
         cluster.sync();
-        all = make_int3(0, 0, 0);
+        all = make_int4(0, 0, 0, 0);
 #pragma unroll
         for (int r = 0; r < CL; ++r) {
-            const int3 o = *cluster.map_shared_rank(&block_total, r);
+            const int4 o = *cluster.map_shared_rank(&block_total, r);
             if (r < rank) {
                 off.x += o.x;
                 off.y += o.y;
                 off.z += o.z;
+                off.w += o.w;
             }
             all.x += o.x;
             all.y += o.y;
             all.z += o.z;
+            all.w += o.w;
         }
         cluster.sync();   // every block has read the totals
     }
     for (int s = s0; s < s1; ++s) {
-        const int3 v = counts(s, c);
-        const int3 ex = warp_exclusive_scan3(v, &tot);
+        const int4 v = counts(s, c);
+        const int4 ex = warp_exclusive_scan4(v, &tot);
         const int t = s * 32 + lane;
         if (next_cnt && t < ntiles) {
             next_bstart[t] = off.z + ex.z;
@@ -870,7 +916,7 @@ __device__ __forceinline__ void plan_body(
             next_cnt[t] = 0;
         }
         const int beg = t < ntiles ? bstart[t] : 0;
-        auto put = [&](int tile, int q, int b0, int fill, int item0, int out0) {
+        auto put = [&](int tile, int q, int b0, int fill, int item0, int out0, int u0) {
             Item it;
             it.tile = tile;
             it.beg = b0 + q * kItem;
@@ -879,23 +925,25 @@ __device__ __forceinline__ void plan_body(
             it.tx = tile % T;
             it.ty = (tile / T) % T;
             it.tz = tile / (T * T);
-            it.pad = 0;
+            it.unit0 = u0 + kUnitTile + q * (kPT * kUnit);
             items[item0 + q] = it;
         };
         // the first items of every tile at once, a lane per tile; what a tile has
         // beyond them by the whole warp, tile by tile
         for (int q = 0; q < min(v.x, kOwnItems); ++q)
-            put(t, q, beg, v.y, off.x + ex.x, off.y + ex.y);
+            put(t, q, beg, v.y, off.x + ex.x, off.y + ex.y, off.w + ex.w);
         for (unsigned left = __ballot_sync(kFull, v.x > kOwnItems); left; left &= left - 1) {
             const int o = __ffs(left) - 1;
             const int n = __shfl_sync(kFull, v.x, o), f = __shfl_sync(kFull, v.y, o);
             const int b0 = __shfl_sync(kFull, beg, o), i0 = off.x + __shfl_sync(kFull, ex.x, o);
             const int o0 = off.y + __shfl_sync(kFull, ex.y, o);
-            for (int q = kOwnItems + lane; q < n; q += 32) put(s * 32 + o, q, b0, f, i0, o0);
+            const int h0 = off.w + __shfl_sync(kFull, ex.w, o);
+            for (int q = kOwnItems + lane; q < n; q += 32) put(s * 32 + o, q, b0, f, i0, o0, h0);
         }
         off.x += tot.x;
         off.y += tot.y;
         off.z += tot.z;
+        off.w += tot.w;
     }
     if (rank != 0) return;
     const int no = *ovf;
@@ -905,11 +953,13 @@ __device__ __forceinline__ void plan_body(
         it.beg = ovf_base + q * kItem;
         it.end = ovf_base + min((q + 1) * kItem, no);
         it.out = all.y + q * kItem;
-        it.tx = it.ty = it.tz = it.pad = 0;
+        it.tx = it.ty = it.tz = 0;
+        it.unit0 = all.w + q * (kPT * kUnit);
         items[all.x + q] = it;
     }
     if (threadIdx.x == 0) {
-        *n_items = all.x + (no + kItem - 1) / kItem;
+        n_items[0] = all.x + (no + kItem - 1) / kItem;
+        n_items[1] = all.w + kUnit * ((no + kNT - 1) / kNT);
         if (next_ovf) *next_ovf = 0;
         if (all.y + no < 0) atomicOr(status, kStatusTotal);
         // scalars of the next step: n + 1 at time t_n = t_{n-1} + dt
@@ -960,7 +1010,7 @@ __global__ void __launch_bounds__(kNT, DepBlock<2>::MIN_BLOCKS)
         sh.dep[i] = 0;
         sh.dep64[i] = 0;
     }
-    const int cnt = threadIdx.x < nruns ? *runs[threadIdx.x].n_items : 0;
+    const int cnt = threadIdx.x < nruns ? runs[threadIdx.x].n_items[0] : 0;
     int total;
     const int ex = block_exclusive_scan(cnt, scan_tmp, &total);
     if (threadIdx.x < nruns) prefix[threadIdx.x] = ex;
@@ -980,10 +1030,10 @@ __global__ void __launch_bounds__(kNT, DepBlock<2>::MIN_BLOCKS)
                             Buf{d.sx[b], d.sy[b], d.sz[b], d.dl[b], d.id[b]},
                             Buf{d.sx[o], d.sy[o], d.sz[o], d.dl[o], d.id[o]},
                             Layout{d.bstart[o], d.cap[o], d.cnt[o], d.ovf[o], d.ovf_base, d.ovf_cap},
-                            d.items, d.acc, d.status, 1, 1};
+                            d.items, d.n_items[0], d.acc, d.status, 1, 1};
         }
         __syncthreads();
-        step_items<2, true>(view, KeysScheduled{view}, lo, hi, sh);
+        step_items<2, kSparse>(view, KeysScheduled{view}, lo, hi, sh);
         __syncthreads();
     }
 }
@@ -1011,10 +1061,14 @@ __global__ void k_plan_flat(int N, Item* items, int* n_items) {
         it.beg = q * kItem;
         it.end = min((q + 1) * kItem, N);
         it.out = q * kItem;
-        it.tx = it.ty = it.tz = it.pad = 0;
+        it.tx = it.ty = it.tz = 0;
+        it.unit0 = q * (kPT * kUnit);
         items[q] = it;
     }
-    if (q == 0) *n_items = nq;
+    if (q == 0) {
+        n_items[0] = nq;
+        n_items[1] = kUnit * ((N + kNT - 1) / kNT);
+    }
 }
 
 // Compacted copy of the live particles (items in order) into `out`.
@@ -1367,26 +1421,40 @@ int step_grid(sipf_ctx* c) {
     int dev = c->device, nsm = 0, per_sm = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (c->p.p2g_order == 4)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<4, false>, kNT, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<4, kDense>, kNT, 0);
     else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<2, false>, kNT, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<2, kDense>, kNT, 0);
     // a tuning may ask for fewer blocks per SM than the occupancy limit
     if (c->step_bps > 0 && c->step_bps < per_sm) per_sm = c->step_bps;
     int g = nsm * (per_sm > 0 ? per_sm : 1);
-    // no more blocks than items can exist: a small run leaves the rest of the
-    // GPU to the runs beside it
+    c->step_blocks_max = g > 0 ? g : 1;
+    // no more blocks than items (or, split, chunks) can exist: a small run leaves
+    // the rest of the GPU to the runs beside it
+    const int64_t chunks = (c->N + kNT - 1) / kNT + c->ntiles;
+    c->split_blocks = static_cast<int>(chunks < c->step_blocks_max ? chunks : c->step_blocks_max);
     if (g > c->max_items) g = c->max_items;
     return g > 0 ? g : 1;
 }
 
 cudaError_t launch_step_kernel(sipf_ctx* c, const PushArgs& a, int do_deposit, int do_move) {
     const int b = c->cur;
-    // runs with fewer than kSparsePerTile particles per tile on average have
-    // many short items: they take the form that skips idle warps
-    const bool sparse = c->N < static_cast<int64_t>(kSparsePerTile) * c->ntiles;
-    auto kernel = c->p.p2g_order == 4 ? (sparse ? k_step<4, true> : k_step<4, false>)
-                                      : (sparse ? k_step<2, true> : k_step<2, false>);
-    return launch_pdl(kernel, dim3(c->step_blocks), dim3(kNT), 0, c->stream, a,
+    // Fewer than kSparsePerTile particles per tile on average: many short items, the
+    // sparse form.  From two chunks per tile on and with fewer full items than
+    // blocks, the split form (32^3 / 2^15: 22.3 -> 18.8 us per step, fourth order
+    // at 64^3 / 2^18 77.5 -> 70.9; with thinner tiles, 72^3 / 2 10^5, it is slower,
+    // 51 against 49 us: two blocks then share a tile that one handles as fast).
+    const int64_t tiles = c->ntiles;
+    const int form = c->N < kSparsePerTile * tiles ? kSparse
+                   : c->N >= 2 * kNT * tiles && c->N < static_cast<int64_t>(kItem) * c->step_blocks_max
+                         ? kSplit : kDense;
+    auto pick = [form](auto dense, auto sparse, auto split) {
+        return form == kSparse ? sparse : form == kSplit ? split : dense;
+    };
+    auto kernel = c->p.p2g_order == 4
+                      ? pick(k_step<4, kDense>, k_step<4, kSparse>, k_step<4, kSplit>)
+                      : pick(k_step<2, kDense>, k_step<2, kSparse>, k_step<2, kSplit>);
+    const int blocks = form == kSplit ? c->split_blocks : c->step_blocks;
+    return launch_pdl(kernel, dim3(blocks), dim3(kNT), 0, c->stream, a,
                       static_cast<const StepScalars*>(c->dsc + b),
                       static_cast<const float4*>(reinterpret_cast<float4*>(c->G)), buf_of(c, b),
                       buf_of(c, b ^ 1), layout_of(c, b ^ 1), static_cast<const Item*>(c->items),

@@ -141,7 +141,7 @@ struct Item {
     int end;
     int out;
     int tx, ty, tz;   // tile coordinates (0 for tile = -1)
-    int pad;
+    int unit0;        // first work unit of its first chunk (particles.cu)
 };
 
 // Spectral-step scalars.
@@ -261,10 +261,12 @@ struct sipf_ctx {
     int* cnt[2] = {nullptr, nullptr};    // arrivals per bucket (incl. overflowed)
     int* ovf[2] = {nullptr, nullptr};    // particles in the overflow region
     sipf::Item* items = nullptr;         // items of the current buffer
-    int* n_items = nullptr;
+    int* n_items = nullptr;              // [2]: items, work units
     int* work = nullptr;                 // work counter of the persistent step kernel
     int max_items = 0;
-    int step_blocks = 0;
+    int step_blocks = 0;                 // blocks of the particle step
+    int step_blocks_max = 1;             // as many as fit on the GPU (or the tuning allows)
+    int split_blocks = 1;                // of its split form
 
     // per-cell histogram (sipf_cell_start)
     int32_t* count = nullptr;        // H^3
