@@ -1258,6 +1258,54 @@ __global__ void k_component(const float4* __restrict__ G, int n, int comp, float
     out[i] = comp == 0 ? g.x : comp == 1 ? g.y : g.z;
 }
 
+// w into the fourth component of the gather array.
+__global__ void k_set_w(const float* __restrict__ w, int n, float* __restrict__ G) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) G[4 * static_cast<size_t>(i) + 3] = w[i];
+}
+
+// What a new state's set-up needs to know of its masses and of v, per block
+// (StateStats; the host folds the blocks).  One pass over both arrays at
+// memory speed.
+constexpr int kStatsBlocks = 304;
+constexpr int kStatsNT = 256;
+
+__global__ void __launch_bounds__(kStatsNT)
+    k_state_stats(const double* __restrict__ mass, int N, const float* __restrict__ v, int n,
+                  StateStats* __restrict__ out) {
+    StateStats s{0.0, LLONG_MAX, 0, 0.0f, INT_MAX, 0};
+    const int stride = kStatsBlocks * kStatsNT;
+    for (int64_t i = blockIdx.x * kStatsNT + threadIdx.x; i < N; i += stride) {
+        const double m = mass[i];
+        if (!(isfinite(m) && m >= 0.0)) {
+            s.flags |= 1;
+        } else {
+            const long long b = __double_as_longlong(m + 0.0);   // -0 counts as 0
+            s.mass_min = b < s.mass_min ? b : s.mass_min;
+            s.mass_max = b > s.mass_max ? b : s.mass_max;
+        }
+    }
+    for (int64_t i = blockIdx.x * kStatsNT + threadIdx.x; i < n; i += stride) {
+        const float x = v[i];
+        const uint32_t b = __float_as_uint(x) & 0x7FFFFFFFu;
+        if (b >= 0x7F800000u) s.flags |= 2;
+        if (b == 0u) continue;
+        const int e = static_cast<int>(b >> 23);
+        const uint32_t man = e ? (b & 0x7FFFFFu) | 0x800000u : b;
+        s.v_low = min(s.v_low, (e ? e - 150 : -149) + __ffs(static_cast<int>(man)) - 1);
+        s.v_max = fmaxf(s.v_max, fabsf(x));
+        s.v_sum += static_cast<double>(x);
+    }
+    __shared__ StateStats part[kStatsNT];
+    part[threadIdx.x] = s;
+    __syncthreads();
+    for (int h = kStatsNT / 2; h > 0; h >>= 1) {
+        if (threadIdx.x < h) part[threadIdx.x].fold(part[threadIdx.x + h]);
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) out[blockIdx.x] = part[0];
+}
+
 // Diagnostics: deterministic two-level reduction (fixed grid, fixed trees).
 // The particle mass is summed exactly, as 128-bit fixed point: each
 // a_p / exp(logref) times 2^K (K chosen on the host so that a term stays
@@ -1638,6 +1686,20 @@ cudaError_t launch_acc_to_float(sipf_ctx* c, float* dst, float scale) {
     const int n = c->H * c->H * c->H;
     k_acc_to_float<<<blocks_for(n, 256), 256, 0, c->stream>>>(
         reinterpret_cast<unsigned long long*>(c->acc), n, scale, dst);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_set_w(sipf_ctx* c) {
+    const int n = c->H * c->H * c->H;
+    k_set_w<<<blocks_for(n, 256), 256, 0, c->stream>>>(c->w, n, c->G);
+    return cudaGetLastError();
+}
+
+int state_stats_blocks() { return kStatsBlocks; }
+
+cudaError_t launch_state_stats(sipf_ctx* c, const double* mass, const float* v, StateStats* out) {
+    k_state_stats<<<kStatsBlocks, kStatsNT, 0, c->stream>>>(mass, static_cast<int>(c->N), v,
+                                                            c->H * c->H * c->H, out);
     return cudaGetLastError();
 }
 

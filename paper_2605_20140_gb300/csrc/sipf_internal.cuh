@@ -144,6 +144,24 @@ struct Item {
     int unit0;        // first work unit of its first chunk (particles.cu)
 };
 
+// Statistics of a state's masses and of v.
+struct StateStats {
+    double v_sum;                 // exact when any_order_exact(n, v_max, v_low)
+    long long mass_min, mass_max; // bits of the smallest and the largest mass
+    float v_max;                  // largest |v|
+    int v_low;                    // every v is a multiple of 2^v_low
+    int flags;                    // 1: a mass is negative or not finite, 2: a v is not finite
+
+    __host__ __device__ void fold(const StateStats& o) {
+        v_sum += o.v_sum;
+        mass_min = o.mass_min < mass_min ? o.mass_min : mass_min;
+        mass_max = o.mass_max > mass_max ? o.mass_max : mass_max;
+        v_max = o.v_max > v_max ? o.v_max : v_max;
+        v_low = o.v_low < v_low ? o.v_low : v_low;
+        flags |= o.flags;
+    }
+};
+
 // Spectral-step scalars.
 struct SpectralArgs {
     float tau;
@@ -292,6 +310,7 @@ struct sipf_ctx {
     float* voff = nullptr;           // device scalar: offset subtracted from v before its FFT
     int kxp = 0;
 
+    double* hstage = nullptr;        // pinned staging of unequal masses (allocated on first use)
     void* rs_scratch = nullptr;      // residual resampling work space (allocated on first use)
     size_t rs_bytes = 0;
 
@@ -353,6 +372,11 @@ cudaError_t launch_iota(sipf_ctx* c, int buf);
 cudaError_t launch_export_mass(sipf_ctx* c, int b, double* out, int as_log);
 cudaError_t launch_acc_to_float(sipf_ctx* c, float* dst, float scale);
 cudaError_t launch_component(sipf_ctx* c, int comp, float* dst);
+cudaError_t launch_set_w(sipf_ctx* c);
+// Per-block statistics of N masses and H^3 values of v (device pointers) into
+// state_stats_blocks() entries at `out`.
+int state_stats_blocks();
+cudaError_t launch_state_stats(sipf_ctx* c, const double* mass, const float* v, StateStats* out);
 cudaError_t launch_diagnostics(sipf_ctx* c, int b, double acc_to_u);
 cudaError_t launch_normals(const uint32_t* ids, int64_t N, uint32_t n, uint64_t seed, float* z,
                            uint32_t* bits, cudaStream_t s);
