@@ -91,30 +91,49 @@ __global__ void k_rs_init(unsigned long long* ext, int* flag) {
 
 // Ids checked, masses a_p = exp(dl + logref) (as exported) in id order,
 // largest and smallest mass (non-negative doubles order like their bits).
-__global__ void k_rs_index(const uint32_t* __restrict__ id, const double* __restrict__ dl,
+__global__ void __launch_bounds__(kRsNT) k_rs_index(const uint32_t* __restrict__ id, const double* __restrict__ dl,
                            double logref, int N, int* __restrict__ perm, double* __restrict__ a,
                            int* seen, unsigned long long* ext, int* flag) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const uint32_t q = id[i];
-    if (q >= static_cast<uint32_t>(N)) {
-        atomicOr(flag, kRsBadId);
-        return;
+    unsigned long long hi = 0ull, lo = ~0ull;
+    if (i < N) {
+        const uint32_t q = id[i];
+        if (q >= static_cast<uint32_t>(N)) {
+            atomicOr(flag, kRsBadId);
+        } else if (atomicAdd(seen + q, 1) != 0) {
+            atomicOr(flag, kRsDupId);
+        } else {
+            perm[q] = i;
+            const double v = exp(dl[i] + logref);
+            a[q] = v;
+            if (!(v >= 0.0) || isinf(v)) atomicOr(flag, kRsNonfinite);
+            else hi = lo = static_cast<unsigned long long>(__double_as_longlong(v));
+        }
     }
-    if (atomicAdd(seen + q, 1) != 0) {
-        atomicOr(flag, kRsDupId);
-        return;
+    // one atomic of each kind per block: for every particle they met on two words
+    // (2^20 particles: 1315 us, of the call's 1.6 ms)
+    __shared__ unsigned long long part[2][kRsNT / 32];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const unsigned long long h = __shfl_xor_sync(0xffffffffu, hi, off);
+        const unsigned long long l = __shfl_xor_sync(0xffffffffu, lo, off);
+        hi = h > hi ? h : hi;
+        lo = l < lo ? l : lo;
     }
-    perm[q] = i;
-    const double v = exp(dl[i] + logref);
-    a[q] = v;
-    if (!(v >= 0.0) || isinf(v)) {
-        atomicOr(flag, kRsNonfinite);
-        return;
+    if ((threadIdx.x & 31) == 0) {
+        part[0][threadIdx.x >> 5] = hi;
+        part[1][threadIdx.x >> 5] = lo;
     }
-    const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(v));
-    atomicMax(ext, b);
-    atomicMin(ext + 1, b);
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int w = 1; w < kRsNT / 32; ++w) {
+        hi = part[0][w] > hi ? part[0][w] : hi;
+        lo = part[1][w] < lo ? part[1][w] : lo;
+    }
+    if (hi >= lo) {   // some particle of the block had a mass
+        atomicMax(ext, hi);
+        atomicMin(ext + 1, lo);
+    }
 }
 
 __device__ __forceinline__ uint64_t q_weight(double a, int E) {
@@ -290,11 +309,11 @@ int resample_device(sipf_ctx* c, int src, int dst, double ratio, int* done, std:
     }
     const RsScratch s = carve(c->rs_scratch, N, tiles);
     cudaStream_t st = c->stream;
-    const int nb = (N + 255) / 256;
+    const int nb = (N + kRsNT - 1) / kRsNT;
     cudaError_t e = cudaMemsetAsync(s.seen, 0, sizeof(int) * N, st);
     if (e == cudaSuccess) {
         k_rs_init<<<1, 1, 0, st>>>(s.ext, s.flag);
-        k_rs_index<<<nb, 256, 0, st>>>(c->id[src], c->dl[src], c->logref, N, s.perm, s.a, s.seen,
+        k_rs_index<<<nb, kRsNT, 0, st>>>(c->id[src], c->dl[src], c->logref, N, s.perm, s.a, s.seen,
                                        s.ext, s.flag);
         e = cudaGetLastError();
     }
