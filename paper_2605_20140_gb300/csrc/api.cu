@@ -343,10 +343,14 @@ int bin_from(sipf_ctx* c, int b) {
     SIPF_CUDA(c, cudaMemsetAsync(c->ovf[b], 0, sizeof(int), c->stream));
     SIPF_CUDA(c, launch_tile_count(c, b, c->cnt[b]));
     SIPF_CUDA(c, launch_plan(c, b, 1, c->stream, 0.0));   // layout of buffer b ^ 1 from the tile counts
-    SIPF_CUDA(c, launch_plan_flat(c));           // items: the raw input array
     c->cur = b;
-    const PushArgs a = push_args(c, 0.0, 0);
-    SIPF_CUDA(c, launch_step_kernel(c, a, 0, 1));
+    if (bins_directly(c)) {
+        SIPF_CUDA(c, launch_bin(c, b));
+    } else {
+        SIPF_CUDA(c, launch_plan_flat(c));       // items: the raw input array
+        const PushArgs a = push_args(c, 0.0, 0);
+        SIPF_CUDA(c, launch_step_kernel(c, a, 0, 1));
+    }
     c->cur = b ^ 1;
     SIPF_CUDA(c, launch_plan(c, b ^ 1, 1, c->stream, 0.0));
     return SIPF_OK;
@@ -790,7 +794,7 @@ int sipf_set_state(sipf_ctx* c, const float* x, const double* mass, const uint32
     }
     int r = SIPF_OK;
     cudaError_t e = launch_wrap_positions(c, px, py, pz, 1);
-    if (e == cudaSuccess) e = launch_rel_log_mass(c, pm, 1);
+    if (e == cudaSuccess) e = launch_rel_log_mass(c, pm, 1, have_mass);
     if (e == cudaSuccess) {
         if (id) {
             r = copy_in(c, c->id[1], id, N * sizeof(uint32_t), where);

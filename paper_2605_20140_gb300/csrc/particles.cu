@@ -1051,6 +1051,65 @@ __global__ void k_tile_count(const float* __restrict__ sx, const float* __restri
     if (t >= 0 && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(cnt + t, __popc(peers));
 }
 
+// The same with the block's counts in shared memory (ntiles of them), added to
+// the grid's once: in a clustered state the particles of one warp after another
+// meet on a few hundred words (128^3 / 2^22: 432 -> 17 us, ncu).
+constexpr int kSharedTiles = 32768;   // 128 KB: H = 256
+constexpr int kBinNT = 512;
+
+__global__ void __launch_bounds__(kBinNT)
+    k_tile_count_shared(const float* __restrict__ sx, const float* __restrict__ sy,
+                        const float* __restrict__ sz, int N, int H, int ntiles,
+                        int* __restrict__ cnt) {
+    extern __shared__ int hist[];
+    for (int t = threadIdx.x; t < ntiles; t += kBinNT) hist[t] = 0;
+    __syncthreads();
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * kBinNT + threadIdx.x; i < N;
+         i += static_cast<int64_t>(gridDim.x) * kBinNT) {
+        const Cell c = locate_clamped(sx[i], sy[i], sz[i], H);
+        atomicAdd(hist + tile_of(c.cx, c.cy, c.cz, H >> 3), 1);
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < ntiles; t += kBinNT)
+        if (hist[t]) atomicAdd(cnt + t, hist[t]);
+}
+
+// Binning of an unbinned array [0, N) into the tile buckets of `dst`: a block
+// counts its share per tile in shared memory, reserves each tile's slots with
+// one global atomic, and hands them out from shared memory on a second pass
+// over its share.  The step kernel's path for unbinned input reserves per warp
+// and tile, about 25 contended atomics a warp (128^3 / 2^22: 488 -> 156 us,
+// ncu); it stays for more tiles than fit.
+__global__ void __launch_bounds__(kBinNT)
+    k_bin(Buf src, Buf dst, Layout L, int N, int H, int ntiles, int* __restrict__ status) {
+    extern __shared__ int slot[];
+    for (int t = threadIdx.x; t < ntiles; t += kBinNT) slot[t] = 0;
+    __syncthreads();
+    const int64_t beg = static_cast<int64_t>(N) * blockIdx.x / gridDim.x;
+    const int64_t end = static_cast<int64_t>(N) * (blockIdx.x + 1) / gridDim.x;
+    for (int64_t i = beg + threadIdx.x; i < end; i += kBinNT) {
+        const Cell c = locate_clamped(src.sx[i], src.sy[i], src.sz[i], H);
+        atomicAdd(slot + tile_of(c.cx, c.cy, c.cz, H >> 3), 1);
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < ntiles; t += kBinNT)
+        if (slot[t]) slot[t] = atomicAdd(L.cnt + t, slot[t]);
+    __syncthreads();
+    for (int64_t i = beg + threadIdx.x; i < end; i += kBinNT) {
+        const float x = src.sx[i], y = src.sy[i], z = src.sz[i];
+        const Cell c = locate_clamped(x, y, z, H);
+        const int t = tile_of(c.cx, c.cy, c.cz, H >> 3);
+        const int k = atomicAdd(slot + t, 1);
+        const int d = k < __ldg(L.cap + t) ? __ldg(L.bstart + t) + k : overflow_slot(L, status);
+        if (d < 0) continue;
+        dst.sx[d] = x;
+        dst.sy[d] = y;
+        dst.sz[d] = z;
+        dst.dl[d] = src.dl[i];
+        dst.id[d] = src.id[i];
+    }
+}
+
 // Whole input as overflow-style items (tile -1) for the initial binning.
 __global__ void k_plan_flat(int N, Item* items, int* n_items) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1218,6 +1277,18 @@ __global__ void k_wrap_positions(const float* __restrict__ x, const float* __res
 __global__ void k_rel_log_mass(const double* __restrict__ mass, int N, double logref, double* dl) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < N) dl[i] = log(mass[i]) - logref;
+}
+
+// The same when every mass is mass[0]: one logarithm per block (float64
+// logarithms of all of 2^22 masses take 237 us).
+__global__ void __launch_bounds__(256)
+    k_rel_log_equal(const double* __restrict__ mass, int N, double logref, double* dl) {
+    __shared__ double v;
+    if (threadIdx.x == 0) v = log(mass[0]) - logref;
+    __syncthreads();
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; i < N;
+         i += static_cast<int64_t>(gridDim.x) * 256)
+        dl[i] = v;
 }
 
 __global__ void k_iota(uint32_t* id, int N) {
@@ -1592,8 +1663,39 @@ RunDesc run_desc(const sipf_ctx* c, double dt) {
     return d;
 }
 
+// Blocks of the kernels that hold a word per tile in shared memory: as many as
+// fit at once (two per SM up to 100 KB), but with at least 2048 particles each.
+static int shared_tile_blocks(sipf_ctx* c, size_t smem) {
+    int nsm = 1;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device);
+    const int64_t fit = nsm * (smem <= 100 * 1024 ? 2 : 1), want = (c->N + 2047) / 2048;
+    return static_cast<int>(want < fit ? want : fit);
+}
+
+bool bins_directly(const sipf_ctx* c) { return c->ntiles <= kSharedTiles; }
+
+cudaError_t launch_bin(sipf_ctx* c, int b) {
+    const size_t smem = static_cast<size_t>(c->ntiles) * sizeof(int);
+    const cudaError_t e = cudaFuncSetAttribute(k_bin, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+    k_bin<<<shared_tile_blocks(c, smem), kBinNT, smem, c->stream>>>(
+        buf_of(c, b), buf_of(c, b ^ 1), layout_of(c, b ^ 1), static_cast<int>(c->N), c->H,
+        c->ntiles, c->status);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_tile_count(sipf_ctx* c, int b, int* cnt) {
     const int N = static_cast<int>(c->N);
+    if (bins_directly(c)) {
+        const size_t smem = static_cast<size_t>(c->ntiles) * sizeof(int);
+        const cudaError_t e = cudaFuncSetAttribute(
+            k_tile_count_shared, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        if (e != cudaSuccess) return e;
+        k_tile_count_shared<<<shared_tile_blocks(c, smem), kBinNT, smem, c->stream>>>(
+            c->sx[b], c->sy[b], c->sz[b], N, c->H, c->ntiles, cnt);
+        return cudaGetLastError();
+    }
     k_tile_count<<<blocks_for(N, 256), 256, 0, c->stream>>>(c->sx[b], c->sy[b], c->sz[b], N, c->H,
                                                              cnt);
     return cudaGetLastError();
@@ -1655,8 +1757,13 @@ cudaError_t launch_wrap_positions(sipf_ctx* c, const float* x, const float* y, c
     return cudaGetLastError();
 }
 
-cudaError_t launch_rel_log_mass(sipf_ctx* c, const double* mass, int buf) {
+cudaError_t launch_rel_log_mass(sipf_ctx* c, const double* mass, int buf, bool equal) {
     const int N = static_cast<int>(c->N);
+    if (equal) {
+        const int nb = blocks_for(N, 256);
+        k_rel_log_equal<<<nb < 1216 ? nb : 1216, 256, 0, c->stream>>>(mass, N, c->logref, c->dl[buf]);
+        return cudaGetLastError();
+    }
     k_rel_log_mass<<<blocks_for(N, 256), 256, 0, c->stream>>>(mass, N, c->logref, c->dl[buf]);
     return cudaGetLastError();
 }

@@ -360,6 +360,10 @@ cudaError_t launch_plan(sipf_ctx* c, int b, int next_layout, cudaStream_t s, dou
 cudaError_t launch_tile_count(sipf_ctx* c, int b, int* cnt);
 cudaError_t launch_plan_flat(sipf_ctx* c);
 cudaError_t launch_compact(sipf_ctx* c, int b, int out);
+// Bins the unbinned particles of buffer b into the buckets of b ^ 1, where
+// bins_directly says that this grid's tiles allow it.
+bool bins_directly(const sipf_ctx* c);
+cudaError_t launch_bin(sipf_ctx* c, int b);
 cudaError_t launch_cell_histogram(sipf_ctx* c, int b, int* count, int* tmp, int* cell_start);
 // cell_start of buffer b and its ids in canonical (cell key, id) order, the
 // latter into b's id array (b's log-masses are overwritten as work space)
@@ -367,7 +371,7 @@ cudaError_t launch_canonical_order(sipf_ctx* c, int b);
 cudaError_t launch_wrap_positions(sipf_ctx* c, const float* x, const float* y, const float* z,
                                   int buf);
 cudaError_t launch_export_positions_inplace(sipf_ctx* c, int b);
-cudaError_t launch_rel_log_mass(sipf_ctx* c, const double* mass, int buf);
+cudaError_t launch_rel_log_mass(sipf_ctx* c, const double* mass, int buf, bool equal);
 cudaError_t launch_iota(sipf_ctx* c, int buf);
 cudaError_t launch_export_mass(sipf_ctx* c, int b, double* out, int as_log);
 cudaError_t launch_acc_to_float(sipf_ctx* c, float* dst, float scale);
