@@ -956,10 +956,8 @@ int sipf_cell_start(sipf_ctx* c, int32_t* cell_start, int where) {
     if (where != SIPF_HOST && where != SIPF_DEVICE) return fail(c, SIPF_EINVAL, "bad where");
     if (!c->state_set) return fail(c, SIPF_EINVAL, "sipf_set_state has not been called");
     const size_t H3 = static_cast<size_t>(c->H) * c->H * c->H;
-    int r = compact_current(c);
-    if (r != SIPF_OK) return r;
-    SIPF_CUDA(c, launch_cell_histogram(c, c->cur ^ 1, c->count, c->scan_tmp, c->cell_start));
-    r = copy_out(c, cell_start, c->cell_start, (H3 + 1) * sizeof(int32_t), where);
+    SIPF_CUDA(c, launch_cell_histogram(c, c->count, c->scan_tmp, c->cell_start));
+    int r = copy_out(c, cell_start, c->cell_start, (H3 + 1) * sizeof(int32_t), where);
     if (r != SIPF_OK) return r;
     return check_status(c);
 }
@@ -1007,8 +1005,7 @@ int sipf_canonical_order(sipf_ctx* c, int32_t* cell_start, uint32_t* ids, int wh
     if (where != SIPF_HOST && where != SIPF_DEVICE) return fail(c, SIPF_EINVAL, "bad where");
     if (!c->state_set) return fail(c, SIPF_EINVAL, "sipf_set_state has not been called");
     const size_t H3 = static_cast<size_t>(c->H) * c->H * c->H;
-    int r = compact_current(c);
-    if (r != SIPF_OK) return r;
+    int r = SIPF_OK;
     const int o = c->cur ^ 1;
     SIPF_CUDA(c, launch_canonical_order(c, o));
     if (cell_start) r = copy_out(c, cell_start, c->cell_start, (H3 + 1) * sizeof(int32_t), where);

@@ -1147,16 +1147,31 @@ __global__ void k_compact(const Item* __restrict__ items, const int* __restrict_
 }
 
 // ------------------------------------------------------------------ per-cell histogram
-__global__ void k_cell_count(const float* __restrict__ sx, const float* __restrict__ sy,
-                             const float* __restrict__ sz, int N, int H, int* __restrict__ count) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t key = 0xffffffffu;
-    if (i < N) {
-        const Cell c = locate_clamped(sx[i], sy[i], sz[i], H);
-        key = cell_key(c.cx, c.cy, c.cz, H >> 3);
+// Particles per cell, from a buffer's items: a block takes one item, whose
+// particles all lie in its tile, counts the tile's 512 cells in shared memory
+// and adds them to the grid's counters once (particles of the overflow items, and any
+// whose position does not match its bucket, one by one).  Per-particle
+// atomics on a clustered state's cells took 141 us at 128^3 / 2^22, this 18.
+constexpr int kCells = kTile * kTile * kTile;
+
+__global__ void __launch_bounds__(kNT)
+    k_cell_count(const Item* __restrict__ items, const int* __restrict__ n_items, Buf src, int H,
+                 int* __restrict__ count) {
+    __shared__ int hist[kCells];
+    if (blockIdx.x >= *n_items) return;
+    const Item it = items[blockIdx.x];
+    for (int l = threadIdx.x; l < kCells; l += kNT) hist[l] = 0;
+    __syncthreads();
+    for (int i = it.beg + threadIdx.x; i < it.end; i += kNT) {
+        const Cell c = locate_clamped(src.sx[i], src.sy[i], src.sz[i], H);
+        const uint32_t key = cell_key(c.cx, c.cy, c.cz, H >> 3);
+        if (static_cast<int>(key >> 9) == it.tile) atomicAdd(hist + (key & 511u), 1);
+        else atomicAdd(count + key, 1);
     }
-    const unsigned peers = __match_any_sync(kFull, key);
-    if (i < N && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(count + key, __popc(peers));
+    __syncthreads();
+    if (it.tile < 0) return;
+    for (int l = threadIdx.x; l < kCells; l += kNT)
+        if (hist[l]) atomicAdd(count + it.tile * kCells + l, hist[l]);
 }
 
 constexpr int kScanNT = 1024;
@@ -1228,20 +1243,52 @@ __global__ void __launch_bounds__(kScanNT) k_scan_apply(const int* __restrict__ 
 // among the ids of its run, which places it at its canonical position.  Ties
 // in id (possible only for caller-given duplicate ids) are broken by slot,
 // so the result is always a permutation.
-__global__ void k_canon_scatter(const float* __restrict__ sx, const float* __restrict__ sy,
-                                const float* __restrict__ sz, const uint32_t* __restrict__ id,
-                                int N, int H, const int* __restrict__ cell_start,
-                                int* __restrict__ fill, uint32_t* __restrict__ keys_tmp,
-                                uint32_t* __restrict__ ids_tmp) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const Cell c = locate_clamped(sx[i], sy[i], sz[i], H);
-    const uint32_t key = cell_key(c.cx, c.cy, c.cz, H >> 3);
-    const int slot = cell_start[key] + atomicAdd(fill + key, 1);
-    keys_tmp[slot] = key;
-    ids_tmp[slot] = id[i];
+// The scatter works on a buffer's items like k_cell_count: the block's counts per
+// cell, one global atomic per cell for its slots, slots handed out from shared
+// memory (one global atomic per particle took 220 us at 128^3 / 2^22, this 51).
+__global__ void __launch_bounds__(kNT)
+    k_canon_scatter(const Item* __restrict__ items, const int* __restrict__ n_items, Buf src, int H,
+                    const int* __restrict__ cell_start, int* __restrict__ fill,
+                    uint32_t* __restrict__ keys_tmp, uint32_t* __restrict__ ids_tmp) {
+    __shared__ int slot[kCells];
+    if (blockIdx.x >= *n_items) return;
+    const Item it = items[blockIdx.x];
+    for (int l = threadIdx.x; l < kCells; l += kNT) slot[l] = 0;
+    __syncthreads();
+    uint32_t keys[kPT];
+#pragma unroll
+    for (int j = 0; j < kPT; ++j) {
+        const int i = it.beg + j * kNT + static_cast<int>(threadIdx.x);
+        keys[j] = 0u;
+        if (i < it.end) {
+            const Cell c = locate_clamped(src.sx[i], src.sy[i], src.sz[i], H);
+            keys[j] = cell_key(c.cx, c.cy, c.cz, H >> 3);
+            if (static_cast<int>(keys[j] >> 9) == it.tile) atomicAdd(slot + (keys[j] & 511u), 1);
+        }
+    }
+    __syncthreads();
+    if (it.tile >= 0)
+        for (int l = threadIdx.x; l < kCells; l += kNT)
+            if (slot[l])
+                slot[l] = cell_start[it.tile * kCells + l] + atomicAdd(fill + it.tile * kCells + l, slot[l]);
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kPT; ++j) {
+        const int i = it.beg + j * kNT + static_cast<int>(threadIdx.x);
+        if (i >= it.end) continue;
+        const uint32_t key = keys[j];
+        const int k = static_cast<int>(key >> 9) == it.tile
+                          ? atomicAdd(slot + (key & 511u), 1)
+                          : cell_start[key] + atomicAdd(fill + key, 1);
+        keys_tmp[k] = key;
+        ids_tmp[k] = src.id[i];
+    }
 }
 
+// Rank of every particle by id inside its cell's run: the run is read in fours
+// where it is aligned (a cell of a dense cloud holds hundreds of particles, and
+// the lanes of a warp mostly read the same run; one at a time 225 us at 128^3 /
+// 2^22, this 423).
 __global__ void k_canon_rank(const uint32_t* __restrict__ keys_tmp,
                              const uint32_t* __restrict__ ids_tmp, int N,
                              const int* __restrict__ cell_start, uint32_t* __restrict__ out) {
@@ -1251,10 +1298,15 @@ __global__ void k_canon_rank(const uint32_t* __restrict__ keys_tmp,
     const int b = cell_start[key], e = cell_start[key + 1];
     const uint32_t me = ids_tmp[j];
     int rank = 0;
-    for (int t = b; t < e; ++t) {
-        const uint32_t o = ids_tmp[t];
-        rank += (o < me) || (o == me && t < j);
+    auto before = [me, j](uint32_t o, int t) { return (o < me) || (o == me && t < j) ? 1 : 0; };
+    const int skew = static_cast<int>((reinterpret_cast<uintptr_t>(ids_tmp) >> 2) & 3u);
+    int t = b;
+    for (; t < e && ((t + skew) & 3); ++t) rank += before(ids_tmp[t], t);
+    for (; t + 4 <= e; t += 4) {
+        const uint4 o = *reinterpret_cast<const uint4*>(ids_tmp + t);
+        rank += before(o.x, t) + before(o.y, t + 1) + before(o.z, t + 2) + before(o.w, t + 3);
     }
+    for (; t < e; ++t) rank += before(ids_tmp[t], t);
     out[b + rank] = me;
 }
 
@@ -1308,17 +1360,28 @@ __global__ void k_export_mass(const double* __restrict__ dl, int N, double logre
     if (i < N) out[i] = as_log ? dl[i] + logref : exp(dl[i] + logref);
 }
 
-// u_bar = acc * scale; the accumulator is cleared for the next deposit.
+// u_bar = acc * scale; the accumulator is cleared for the next deposit.  PER
+// nodes per thread: two when the output allows float2 stores (16-byte loads and
+// stores of the accumulator).
+template <int PER>
 __global__ void k_acc_to_float(unsigned long long* __restrict__ acc, int n, float scale,
                                float* __restrict__ out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) * PER;
     if (i >= n) return;
-    const unsigned long long q = acc[i];
-    acc[i] = 0ull;
     // two's complement: signed high half, unsigned low half
-    const float f = fmaf(__int2float_rn(static_cast<int>(static_cast<unsigned>(q >> 32))),
-                         4294967296.0f, __uint2float_rn(static_cast<unsigned>(q)));
-    out[i] = f * scale;
+    auto value = [scale](unsigned long long q) {
+        return fmaf(__int2float_rn(static_cast<int>(static_cast<unsigned>(q >> 32))), 4294967296.0f,
+                    __uint2float_rn(static_cast<unsigned>(q))) * scale;
+    };
+    if constexpr (PER == 2) {
+        const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(acc + i);
+        *reinterpret_cast<ulonglong2*>(acc + i) = make_ulonglong2(0ull, 0ull);
+        *reinterpret_cast<float2*>(out + i) = make_float2(value(q.x), value(q.y));
+    } else {
+        const unsigned long long q = acc[i];
+        acc[i] = 0ull;
+        out[i] = value(q);
+    }
 }
 
 // One component of the interleaved (dv/dx, dv/dy, dv/dz, w) array.
@@ -1714,14 +1777,13 @@ cudaError_t launch_compact(sipf_ctx* c, int b, int out) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_cell_histogram(sipf_ctx* c, int b, int* count, int* tmp, int* cell_start) {
-    const int N = static_cast<int>(c->N);
+cudaError_t launch_cell_histogram(sipf_ctx* c, int* count, int* tmp, int* cell_start) {
     const int n = c->H * c->H * c->H;
     const int ntiles = (n + kScanTile - 1) / kScanTile;
     cudaError_t e = cudaMemsetAsync(count, 0, static_cast<size_t>(n) * sizeof(int), c->stream);
     if (e != cudaSuccess) return e;
-    k_cell_count<<<blocks_for(N, 256), 256, 0, c->stream>>>(c->sx[b], c->sy[b], c->sz[b], N, c->H,
-                                                             count);
+    k_cell_count<<<c->max_items, kNT, 0, c->stream>>>(c->items, c->n_items, buf_of(c, c->cur), c->H,
+                                                      count);
     k_scan_tiles<<<ntiles, kScanNT, 0, c->stream>>>(count, n, tmp);
     k_scan_tile_sums<<<1, kScanNT, 0, c->stream>>>(tmp, ntiles, cell_start, n);
     k_scan_apply<<<ntiles, kScanNT, 0, c->stream>>>(count, n, tmp, cell_start);
@@ -1731,17 +1793,17 @@ cudaError_t launch_cell_histogram(sipf_ctx* c, int b, int* count, int* tmp, int*
 cudaError_t launch_canonical_order(sipf_ctx* c, int b) {
     const int N = static_cast<int>(c->N);
     const int n = c->H * c->H * c->H;
-    cudaError_t e = launch_cell_histogram(c, b, c->count, c->scan_tmp, c->cell_start);
+    cudaError_t e = launch_cell_histogram(c, c->count, c->scan_tmp, c->cell_start);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(c->count, 0, static_cast<size_t>(n) * sizeof(int), c->stream);
     if (e != cudaSuccess) return e;
-    // the buffer's log-mass array (8 N bytes) holds the keys and ids of the
-    // counting sort; the ranked ids go to the buffer's id array
+    // the free buffer's log-mass array (8 N bytes) holds the keys and ids of the
+    // counting sort; the ranked ids go to its id array
     uint32_t* keys_tmp = reinterpret_cast<uint32_t*>(c->dl[b]);
     uint32_t* ids_tmp = keys_tmp + N;
-    k_canon_scatter<<<blocks_for(N, 256), 256, 0, c->stream>>>(
-        c->sx[b], c->sy[b], c->sz[b], c->id[b], N, c->H, c->cell_start, c->count, keys_tmp,
-        ids_tmp);
+    k_canon_scatter<<<c->max_items, kNT, 0, c->stream>>>(c->items, c->n_items, buf_of(c, c->cur),
+                                                         c->H, c->cell_start, c->count, keys_tmp,
+                                                         ids_tmp);
     k_canon_rank<<<blocks_for(N, 256), 256, 0, c->stream>>>(keys_tmp, ids_tmp, N, c->cell_start,
                                                             c->id[b]);
     return cudaGetLastError();
@@ -1791,8 +1853,11 @@ cudaError_t launch_export_mass(sipf_ctx* c, int b, double* out, int as_log) {
 
 cudaError_t launch_acc_to_float(sipf_ctx* c, float* dst, float scale) {
     const int n = c->H * c->H * c->H;
-    k_acc_to_float<<<blocks_for(n, 256), 256, 0, c->stream>>>(
-        reinterpret_cast<unsigned long long*>(c->acc), n, scale, dst);
+    unsigned long long* acc = reinterpret_cast<unsigned long long*>(c->acc);
+    if (reinterpret_cast<uintptr_t>(dst) % 8 == 0)   // n is even
+        k_acc_to_float<2><<<blocks_for(n / 2, 256), 256, 0, c->stream>>>(acc, n, scale, dst);
+    else
+        k_acc_to_float<1><<<blocks_for(n, 256), 256, 0, c->stream>>>(acc, n, scale, dst);
     return cudaGetLastError();
 }
 

@@ -364,9 +364,10 @@ cudaError_t launch_compact(sipf_ctx* c, int b, int out);
 // bins_directly says that this grid's tiles allow it.
 bool bins_directly(const sipf_ctx* c);
 cudaError_t launch_bin(sipf_ctx* c, int b);
-cudaError_t launch_cell_histogram(sipf_ctx* c, int b, int* count, int* tmp, int* cell_start);
-// cell_start of buffer b and its ids in canonical (cell key, id) order, the
-// latter into b's id array (b's log-masses are overwritten as work space)
+cudaError_t launch_cell_histogram(sipf_ctx* c, int* count, int* tmp, int* cell_start);
+// cell_start of the current buffer and its ids in canonical (cell key, id)
+// order, the latter into the id array of the free buffer b (whose log-masses
+// are overwritten as work space)
 cudaError_t launch_canonical_order(sipf_ctx* c, int b);
 cudaError_t launch_wrap_positions(sipf_ctx* c, const float* x, const float* y, const float* z,
                                   int buf);
