@@ -1285,10 +1285,10 @@ __global__ void __launch_bounds__(kNT)
     }
 }
 
-// Rank of every particle by id inside its cell's run: the run is read in fours
-// where it is aligned (a cell of a dense cloud holds hundreds of particles, and
-// the lanes of a warp mostly read the same run; one at a time 225 us at 128^3 /
-// 2^22, this 423).
+// Rank of every particle by id inside its cell's run.  The lanes of a warp
+// mostly read the same run, so each read is one broadcast (225 us at 128^3 /
+// 2^22, whose dense cells hold hundreds of particles; reading the run in fours
+// behind an unaligned head took 423).
 __global__ void k_canon_rank(const uint32_t* __restrict__ keys_tmp,
                              const uint32_t* __restrict__ ids_tmp, int N,
                              const int* __restrict__ cell_start, uint32_t* __restrict__ out) {
@@ -1298,15 +1298,10 @@ __global__ void k_canon_rank(const uint32_t* __restrict__ keys_tmp,
     const int b = cell_start[key], e = cell_start[key + 1];
     const uint32_t me = ids_tmp[j];
     int rank = 0;
-    auto before = [me, j](uint32_t o, int t) { return (o < me) || (o == me && t < j) ? 1 : 0; };
-    const int skew = static_cast<int>((reinterpret_cast<uintptr_t>(ids_tmp) >> 2) & 3u);
-    int t = b;
-    for (; t < e && ((t + skew) & 3); ++t) rank += before(ids_tmp[t], t);
-    for (; t + 4 <= e; t += 4) {
-        const uint4 o = *reinterpret_cast<const uint4*>(ids_tmp + t);
-        rank += before(o.x, t) + before(o.y, t + 1) + before(o.z, t + 2) + before(o.w, t + 3);
+    for (int t = b; t < e; ++t) {
+        const uint32_t o = ids_tmp[t];
+        rank += (o < me) || (o == me && t < j);
     }
-    for (; t < e; ++t) rank += before(ids_tmp[t], t);
     out[b + rank] = me;
 }
 
