@@ -1018,10 +1018,9 @@ int sipf_canonical_order(sipf_ctx* c, int32_t* cell_start, uint32_t* ids, int wh
 int sipf_diagnostics(sipf_ctx* c, sipf_diag* out) {
     if (!c || !out) return SIPF_EINVAL;
     if (!c->state_set) return fail(c, SIPF_EINVAL, "sipf_set_state has not been called");
-    int r = compact_current(c);
-    if (r == SIPF_OK) r = deposit_current(c);
+    const int r = deposit_current(c);
     if (r != SIPF_OK) return r;
-    SIPF_CUDA(c, launch_diagnostics(c, c->cur ^ 1, acc_to_u_d(c)));
+    SIPF_CUDA(c, launch_diagnostics(c, acc_to_u_d(c)));
     const size_t H3 = static_cast<size_t>(c->H) * c->H * c->H;
     SIPF_CUDA(c, cudaMemsetAsync(c->acc, 0, H3 * sizeof(long long), c->stream));
     double h[8];

@@ -1285,22 +1285,42 @@ __global__ void __launch_bounds__(kNT)
     }
 }
 
-// Rank of every particle by id inside its cell's run.  The lanes of a warp
-// mostly read the same run, so each read is one broadcast (225 us at 128^3 /
-// 2^22, whose dense cells hold hundreds of particles; reading the run in fours
-// behind an unaligned head took 423).
-__global__ void k_canon_rank(const uint32_t* __restrict__ keys_tmp,
-                             const uint32_t* __restrict__ ids_tmp, int N,
-                             const int* __restrict__ cell_start, uint32_t* __restrict__ out) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= N) return;
+// Rank of every particle by id inside its cell's run.  A block of consecutive
+// places brings the runs it touches into shared memory (a dense cell of 128^3 /
+// 2^22 holds hundreds of particles, so they are little more than the block's own
+// places) and each thread reads its run there, the lanes of a warp mostly the same
+// one; runs that do not fit are read from global memory.  A tie counts for the
+// places before j only, so the loop is split there.  225 -> 194 us at 128^3 / 2^22
+// (ncu), bound by the 10^9 comparisons.
+constexpr int kRankNT = 256;
+constexpr int kRankIds = 2560;
+
+__global__ void __launch_bounds__(kRankNT)
+    k_canon_rank(const uint32_t* __restrict__ keys_tmp, const uint32_t* __restrict__ ids_tmp, int N,
+                 const int* __restrict__ cell_start, uint32_t* __restrict__ out) {
+    __shared__ uint32_t ids[kRankIds];
+    const int j0 = blockIdx.x * kRankNT, j1 = min(j0 + kRankNT, N) - 1;
+    const int lo = cell_start[keys_tmp[j0]], hi = cell_start[keys_tmp[j1] + 1];
+    const bool held = hi - lo <= kRankIds;
+    if (held)
+        for (int t = threadIdx.x; t < hi - lo; t += kRankNT) ids[t] = ids_tmp[lo + t];
+    __syncthreads();
+    const int j = j0 + static_cast<int>(threadIdx.x);
+    if (j > j1) return;
     const uint32_t key = keys_tmp[j];
     const int b = cell_start[key], e = cell_start[key + 1];
-    const uint32_t me = ids_tmp[j];
     int rank = 0;
-    for (int t = b; t < e; ++t) {
-        const uint32_t o = ids_tmp[t];
-        rank += (o < me) || (o == me && t < j);
+    uint32_t me;
+    if (held) {
+        me = ids[j - lo];
+#pragma unroll 8
+        for (int t = b - lo; t < j - lo; ++t) rank += ids[t] <= me;
+#pragma unroll 8
+        for (int t = j - lo + 1; t < e - lo; ++t) rank += ids[t] < me;
+    } else {
+        me = ids_tmp[j];
+        for (int t = b; t < j; ++t) rank += ids_tmp[t] <= me;
+        for (int t = j + 1; t < e; ++t) rank += ids_tmp[t] < me;
     }
     out[b + rank] = me;
 }
@@ -1446,8 +1466,7 @@ constexpr int kDiagNT = 256;
 __device__ __forceinline__ double dmin(double a, double b) { return a < b ? a : b; }
 
 __global__ void __launch_bounds__(kDiagNT)
-    k_diag_partials(const double* __restrict__ dl, double logref, const float* __restrict__ sx,
-                    const float* __restrict__ sy, const float* __restrict__ sz, int N,
+    k_diag_partials(const Item* __restrict__ items, const int* __restrict__ n_items, Buf src,
                     const float* __restrict__ v, const float* __restrict__ m,
                     const float* __restrict__ w, const unsigned long long* __restrict__ acc,
                     int ncell, int K, double* __restrict__ part_d, long long* __restrict__ part_l) {
@@ -1455,9 +1474,15 @@ __global__ void __launch_bounds__(kDiagNT)
     unsigned __int128 mass = 0;
     long long as = 0, amin = LLONG_MAX;
     const int stride = kDiagBlocks * kDiagNT;
-    for (int i = blockIdx.x * kDiagNT + threadIdx.x; i < N; i += stride) {
-        mass += __double2ull_rn(scalbn(exp(dl[i]), K));
-        if (!isfinite(sx[i]) || !isfinite(sy[i]) || !isfinite(sz[i])) nf += 1.0;
+    // particles where they lie in the buckets, item by item (a compact copy of them
+    // first took 58 us at 2^22)
+    const int n = *n_items;
+    for (int q = blockIdx.x; q < n; q += kDiagBlocks) {
+        const int end = items[q].end;
+        for (int i = items[q].beg + threadIdx.x; i < end; i += kDiagNT) {
+            mass += __double2ull_rn(scalbn(exp(src.dl[i]), K));
+            if (!isfinite(src.sx[i]) || !isfinite(src.sy[i]) || !isfinite(src.sz[i])) nf += 1.0;
+        }
     }
     for (int i = blockIdx.x * kDiagNT + threadIdx.x; i < ncell; i += stride) {
         const float a = v[i], b = m[i], c = w[i];
@@ -1799,7 +1824,7 @@ cudaError_t launch_canonical_order(sipf_ctx* c, int b) {
     k_canon_scatter<<<c->max_items, kNT, 0, c->stream>>>(c->items, c->n_items, buf_of(c, c->cur),
                                                          c->H, c->cell_start, c->count, keys_tmp,
                                                          ids_tmp);
-    k_canon_rank<<<blocks_for(N, 256), 256, 0, c->stream>>>(keys_tmp, ids_tmp, N, c->cell_start,
+    k_canon_rank<<<blocks_for(N, kRankNT), kRankNT, 0, c->stream>>>(keys_tmp, ids_tmp, N, c->cell_start,
                                                             c->id[b]);
     return cudaGetLastError();
 }
@@ -1877,14 +1902,14 @@ cudaError_t launch_component(sipf_ctx* c, int comp, float* dst) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_diagnostics(sipf_ctx* c, int b, double acc_to_u) {
+cudaError_t launch_diagnostics(sipf_ctx* c, double acc_to_u) {
     // a_p / exp(logref) <= maxrel e^time (growth factor of a step < e^tau)
     const double bound = log2(c->maxrel) + c->time * 1.4426950408889634 + 1.0;
     int K = 61 - static_cast<int>(ceil(bound));
     K = K < -900 ? -900 : (K > 900 ? 900 : K);
     k_diag_partials<<<kDiagBlocks, kDiagNT, 0, c->stream>>>(
-        c->dl[b], c->logref, c->sx[b], c->sy[b], c->sz[b], static_cast<int>(c->N), c->v, c->m,
-        c->w, reinterpret_cast<const unsigned long long*>(c->acc), c->H * c->H * c->H, K,
+        c->items, c->n_items, buf_of(c, c->cur), c->v, c->m, c->w,
+        reinterpret_cast<const unsigned long long*>(c->acc), c->H * c->H * c->H, K,
         c->diag_tmp, c->diag_ll);
     k_diag_final<<<1, kDiagFinalNT, 0, c->stream>>>(c->diag_tmp, c->diag_ll, acc_to_u, K, c->logref,
                                           c->diag_out);

@@ -382,7 +382,7 @@ cudaError_t launch_set_w(sipf_ctx* c);
 // state_stats_blocks() entries at `out`.
 int state_stats_blocks();
 cudaError_t launch_state_stats(sipf_ctx* c, const double* mass, const float* v, StateStats* out);
-cudaError_t launch_diagnostics(sipf_ctx* c, int b, double acc_to_u);
+cudaError_t launch_diagnostics(sipf_ctx* c, double acc_to_u);
 cudaError_t launch_normals(const uint32_t* ids, int64_t N, uint32_t n, uint64_t seed, float* z,
                            uint32_t* bits, cudaStream_t s);
 // Batched particle kernels of an ensemble whose n <= kMaxRuns members all
