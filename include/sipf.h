@@ -193,8 +193,9 @@ int sipf_canonical_order(sipf_ctx* ctx, int32_t* cell_start, uint32_t* ids, int 
 /* Tuning.  Launch choices that change speed, never results beyond float32
  * rounding: radix_plan selects how the spectral step transforms: 0 or 1,
  * two Stockham plans of each transform length in the plane passes (e.g.
- * 96 = 8 x 4 x 3 or 12 x 8); 2, the per-axis pipeline of transforms held by
- * groups of lanes (H = 64, 128, 256; other sizes take plan 0 instead); the
+ * 96 = 8 x 4 x 3 or 12 x 8); 2, the per-axis passes, which grids above 128
+ * always take, in a variant for H = 64, 128, 256 (other sizes take plan 0
+ * instead); the
  * plans' results differ only by float32 rounding;
  * step_blocks_per_sm (0 = the occupancy limit, else at
  * most that many particle-step blocks per SM); bucket capacity = count +

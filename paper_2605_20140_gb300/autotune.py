@@ -3,7 +3,7 @@
 For each target (grid size H, a particle-count class [N_min, N_max] and a
 representative N), it times every candidate tuning (radix plan of the
 spectral passes: two Stockham plans of the plane passes, or the per-axis
-pipeline of lane-group transforms; particle-step blocks per SM; bucket
+passes; particle-step blocks per SM; bucket
 slack) on the GPU:
 the seeded workload of that size is set up, the tuning applied, a few
 warm-up steps taken, and `steps` steps timed with CUDA events on the
@@ -33,7 +33,7 @@ if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
 RADIX_PLANS = (0, 1, 2)
-WARP_PIPELINE_H = (64, 128, 256)             # grid sizes with radix plan 2
+AXIS_PASSES_H = (64, 128, 256)             # grid sizes with radix plan 2
 STEP_BLOCKS = (0, 4, 3)                      # 0: the occupancy limit
 SLACKS = ((8, 32), (16, 16), (32, 8))        # (bucket_slack_div, bucket_slack_add)
 
@@ -49,7 +49,7 @@ for _H in (32, 48, 64, 96):
 
 def candidates(H=None):
     """Candidate tunings (for grid size H: without plan 2 where H has none)."""
-    plans = [p for p in RADIX_PLANS if p != 2 or H is None or H in WARP_PIPELINE_H]
+    plans = [p for p in RADIX_PLANS if p != 2 or H is None or H in AXIS_PASSES_H]
     return [dict(radix_plan=p, step_blocks_per_sm=b, bucket_slack_div=d, bucket_slack_add=a)
             for p, b, (d, a) in itertools.product(plans, STEP_BLOCKS, SLACKS)]
 

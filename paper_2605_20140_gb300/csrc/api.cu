@@ -592,6 +592,7 @@ int create_in_pool(const sipf_grid* grid, int64_t N, const sipf_params* params,
     if (c->p.p2g_order == 0) c->p.p2g_order = 2;
     c->stream = stream;
     c->pool = pool;
+    c->beside_others = pool != nullptr;
     cudaGetDevice(&c->device);
     const CtxSizes z = ctx_sizes(c->H, N);
     const size_t H3 = z.H3, spec = z.spec;
@@ -1509,6 +1510,7 @@ int sipf_ensemble_create(int32_t count, const sipf_grid* grids, const int64_t* N
             ensemble_free(e);
             return r;
         }
+        c->beside_others = true;
         e->members.push_back(c);
         cudaEvent_t ev = nullptr;
         if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {

@@ -1645,9 +1645,13 @@ cudaError_t launch_step_kernel(sipf_ctx* c, const PushArgs& a, int do_deposit, i
     // blocks, the split form (32^3 / 2^15: 22.3 -> 18.8 us per step, fourth order
     // at 64^3 / 2^18 77.5 -> 70.9; with thinner tiles, 72^3 / 2 10^5, it is slower,
     // 51 against 49 us: two blocks then share a tile that one handles as fast).
+    // Runs beside others (served requests, ensemble members on streams of their
+    // own) stay dense: there the SMs' time counts, and split shares enter more
+    // tiles (eight requests of 400 steps 77 ms split, 73 dense).
     const int64_t tiles = c->ntiles;
     const int form = c->N < kSparsePerTile * tiles ? kSparse
-                   : c->N >= 2 * kNT * tiles && c->N < static_cast<int64_t>(kItem) * c->step_blocks_max
+                   : !c->beside_others && c->N >= 2 * kNT * tiles &&
+                             c->N < static_cast<int64_t>(kItem) * c->step_blocks_max
                          ? kSplit : kDense;
     auto pick = [form](auto dense, auto sparse, auto split) {
         return form == kSparse ? sparse : form == kSplit ? split : dense;

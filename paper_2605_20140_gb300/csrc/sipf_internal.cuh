@@ -260,6 +260,7 @@ struct sipf_ctx {
     int step_bps = 0;
     int slack_div = 8;
     int slack_add = 32;
+    bool beside_others = false;          // shares the GPU with other contexts (server, ensemble)
     cudaMemPool_t pool = nullptr;        // stream-ordered allocation from this pool (null: cudaMalloc)
 
     // particle store, ping-pong; positions in grid units, log-mass relative
