@@ -837,9 +837,9 @@ int sipf_set_state(sipf_ctx* c, const float* x, const double* mass, const uint32
     if (e == cudaSuccess && r == SIPF_OK) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "sipf_set_state");
     if (r != SIPF_OK) return r;
-    r = check_status(c);
+    r = write_scalars(c);   // also of a state whose non-finite positions were reset
     if (r != SIPF_OK) return r;
-    r = write_scalars(c);
+    r = check_status(c);
     if (r != SIPF_OK) return r;
     c->state_set = true;
     return SIPF_OK;

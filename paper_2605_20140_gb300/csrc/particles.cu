@@ -839,8 +839,7 @@ __device__ __forceinline__ void plan_body(
     const int* __restrict__ bstart, const int* __restrict__ ovf, int ovf_base, Item* items,
     int* n_items, int* next_bstart, int* next_cap, int* next_cnt, int* next_ovf,
     int* __restrict__ status, const StepScalars* __restrict__ cur_sc,
-    StepScalars* __restrict__ next_sc, double dt, double log2_maxrel, double exp_logref,
-    double h3, int slack_div, int slack_add) {
+    StepScalars* __restrict__ next_sc, double dt, double h3, int slack_div, int slack_add) {
     constexpr int NW = kPlanNT / 32;
     constexpr int kOwnItems = 4;
     __shared__ int4 warp_base[NW];
@@ -964,8 +963,8 @@ __device__ __forceinline__ void plan_body(
         if (all.y + no < 0) atomicOr(status, kStatusTotal);
         // scalars of the next step: n + 1 at time t_n = t_{n-1} + dt
         if (next_sc)
-            fill_step_scalars(next_sc, cur_sc->n + 1u, cur_sc->time + dt, log2_maxrel, exp_logref,
-                              h3);
+            fill_step_scalars(next_sc, cur_sc->n + 1u, cur_sc->time + dt, cur_sc->log2_maxrel,
+                              cur_sc->exp_logref, h3);
     }
 }
 
@@ -975,11 +974,9 @@ __global__ void __launch_bounds__(kPlanNT)
            const int* __restrict__ bstart, const int* __restrict__ ovf, int ovf_base, Item* items,
            int* n_items, int* next_bstart, int* next_cap, int* next_cnt, int* next_ovf,
            int* __restrict__ status, const StepScalars* __restrict__ cur_sc,
-           StepScalars* __restrict__ next_sc, double dt, double log2_maxrel, double exp_logref,
-           double h3, int slack_div, int slack_add) {
+           StepScalars* __restrict__ next_sc, double dt, double h3, int slack_div, int slack_add) {
     plan_body<CL>(ntiles, T, cnt, cap, bstart, ovf, ovf_base, items, n_items, next_bstart, next_cap,
-                  next_cnt, next_ovf, status, cur_sc, next_sc, dt, log2_maxrel, exp_logref, h3,
-                  slack_div, slack_add);
+                  next_cnt, next_ovf, status, cur_sc, next_sc, dt, h3, slack_div, slack_add);
 }
 
 // The plan of every run of an ensemble after a batched step from buffer
@@ -991,7 +988,7 @@ __global__ void __launch_bounds__(kPlanNT) k_plan_multi(const RunDesc* __restric
     const int b = parity ^ 1, o = parity;
     plan_body<1>(d.ntiles, d.H / 8, d.cnt[b], d.cap[b], d.bstart[b], d.ovf[b], d.ovf_base, d.items,
               d.n_items, d.bstart[o], d.cap[o], d.cnt[o], d.ovf[o], d.status, d.dsc + o,
-              d.dsc + b, d.dt, d.log2_maxrel, d.exp_logref, d.h3, d.slack_div, d.slack_add);
+              d.dsc + b, d.dt, d.h3, d.slack_div, d.slack_add);
 }
 
 // One persistent launch over the items of all runs of an ensemble (all
@@ -1694,7 +1691,7 @@ cudaError_t launch_plan(sipf_ctx* c, int b, int next_layout, cudaStream_t s, dou
         next_layout ? c->ovf[o] : nullptr, c->status,
         // b is the buffer the step just wrote: its slot is the next step's, o's the current one
         static_cast<const StepScalars*>(c->dsc + o), dt > 0.0 ? c->dsc + b : nullptr, dt,
-        c->log2_maxrel, c->exp_logref, c->h3, c->slack_div, c->slack_add);
+        c->h3, c->slack_div, c->slack_add);
 }
 
 cudaError_t launch_step_multi(const RunDesc* runs, int n, int parity, cudaStream_t s) {
@@ -1742,8 +1739,6 @@ RunDesc run_desc(const sipf_ctx* c, double dt) {
     d.status = c->status;
     d.dsc = c->dsc;
     d.dt = dt;
-    d.log2_maxrel = c->log2_maxrel;
-    d.exp_logref = c->exp_logref;
     d.h3 = c->h3;
     d.slack_div = c->slack_div;
     d.slack_add = c->slack_add;

@@ -98,7 +98,9 @@ struct PushArgs {
 // Per-step scalars, kept in device memory (one slot per buffer parity) so
 // that the kernels of a step read them there rather than as launch
 // arguments: the plan kernel of step n writes step n + 1's slot, and a
-// captured sequence of steps can be replayed.
+// captured sequence of steps can be replayed.  The state's mass reference is
+// handed on from slot to slot too, so that a captured sequence holds nothing of the
+// state it was captured with (another state of the context has another reference).
 struct StepScalars {
     uint32_t n;            // the step being taken (Philox counter word 0), from 1
     int32_t deposit_shift; // S of deposit_scale = 2^S
@@ -106,6 +108,8 @@ struct StepScalars {
     float deposit_scale;   // 2^S: contribution of a particle to a node is
                            // exp(log a - logref) * weight * 2^S, rounded to an integer
     float u_scale;         // u_bar per accumulator unit: 2^-S exp(logref) / h^3
+    double log2_maxrel;    // of the state: log2(max_p a_p(0) / exp(logref))
+    double exp_logref;     // of the state: exp(logref)
 };
 
 // S for the deposit at time t: one contribution is at most
@@ -130,6 +134,8 @@ __host__ __device__ inline void fill_step_scalars(StepScalars* s, uint32_t n, do
     s->time = t;
     s->deposit_scale = static_cast<float>(ldexp(1.0, S));
     s->u_scale = static_cast<float>(ldexp(exp_logref, -S) / h3);
+    s->log2_maxrel = log2_maxrel;
+    s->exp_logref = exp_logref;
 }
 
 // A run of particles read by one block of the step kernel: [beg, end) of a
@@ -233,7 +239,7 @@ struct RunDesc {
     const float* G;
     int* status;
     StepScalars* dsc;                   // [2], slot = parity of the source buffer
-    double dt, log2_maxrel, exp_logref, h3;
+    double dt, h3;
     int slack_div, slack_add;           // bucket capacity count + count/slack_div + slack_add
 };
 constexpr int kMaxRuns = 256;           // runs of one batched particle launch
