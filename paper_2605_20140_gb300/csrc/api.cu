@@ -970,6 +970,7 @@ int sipf_set_tuning(sipf_ctx* c, const sipf_tuning* t) {
     cudaStreamSynchronize(c->stream);
     for (const auto& g : c->graphs) cudaGraphExecDestroy(g.exec);
     c->graphs.clear();
+    c->tunings += 1;
     apply_tuning(c, *t);
     c->step_blocks = step_grid(c);
     return SIPF_OK;
@@ -1266,6 +1267,7 @@ struct sipf_ensemble {
     struct BatchGraph {
         std::vector<double> dt;
         int parity;
+        uint64_t tunings;                // of the members at its capture (member_tunings)
         cudaGraphExec_t exec;
         sipf::RunDesc* d_runs;
     };
@@ -1377,15 +1379,25 @@ int enqueue_batched_step(sipf_ensemble* e, const double* dt, const RunDesc* d_ru
     return SIPF_OK;
 }
 
-// The two-step graph of the current parity and dt vector (captured on the
-// first call), with its run table.
+// How often the members' tunings have been set, in all: a graph and its run table
+// hold the members' radix plans and bucket slack, so they serve only while this
+// stays (each member's count only grows).
+uint64_t member_tunings(const sipf_ensemble* e) {
+    uint64_t n = 0;
+    for (const sipf_ctx* c : e->members) n += c->tunings;
+    return n;
+}
+
+// The two-step graph of the current parity, dt vector and tunings (captured on
+// the first call), with its run table.
 int batched_graph(sipf_ensemble* e, const double* dt, sipf_ensemble::BatchGraph** out) {
     *out = nullptr;
     const size_t n = e->members.size();
     const int parity = e->members[0]->cur;
     std::vector<double> dts(dt, dt + n);
+    const uint64_t tunings = member_tunings(e);
     for (auto& g : e->graphs)
-        if (g.parity == parity && g.dt == dts) {
+        if (g.parity == parity && g.tunings == tunings && g.dt == dts) {
             *out = &g;
             return SIPF_OK;
         }
@@ -1437,7 +1449,7 @@ int batched_graph(sipf_ensemble* e, const double* dt, sipf_ensemble::BatchGraph*
         cudaFree(e->graphs.front().d_runs);
         e->graphs.erase(e->graphs.begin());
     }
-    e->graphs.push_back({dts, parity, exec, d_runs});
+    e->graphs.push_back({dts, parity, tunings, exec, d_runs});
     *out = &e->graphs.back();
     return SIPF_OK;
 }

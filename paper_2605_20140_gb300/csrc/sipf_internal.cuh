@@ -266,6 +266,7 @@ struct sipf_ctx {
     int step_bps = 0;
     int slack_div = 8;
     int slack_add = 32;
+    uint64_t tunings = 0;                // calls of sipf_set_tuning (an ensemble's graphs hold the choices)
     bool beside_others = false;          // shares the GPU with other contexts (server, ensemble)
     cudaMemPool_t pool = nullptr;        // stream-ordered allocation from this pool (null: cudaMalloc)
 
