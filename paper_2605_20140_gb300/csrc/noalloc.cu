@@ -193,8 +193,10 @@ __global__ void __launch_bounds__(kNaNT)
 constexpr int kSlabNT = 512;
 constexpr int kScan = 4;        // z read per thread and round
 
+constexpr int kSlabBytes = 200 * 1024;   // a slab's node sums at most, eight bytes each
+
 __host__ __device__ inline int na_slab_planes(int H) {   // planes per slab, one more is held
-    const int p = 200 * 1024 / (H * H * 8) - 1;
+    const int p = kSlabBytes / (H * H * 8) - 1;
     return p < H ? p : H;
 }
 
@@ -389,8 +391,9 @@ extern "C" int sipf_deposit_noalloc(const sipf_grid* grid, const float* x, const
             e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         const size_t smem = static_cast<size_t>(na_slab_planes(H) + 1) * H * H * 2 * sizeof(uint32_t);
         if (e == cudaSuccess)
+            // the limit belongs to the kernel, not to this call: the same for every H
             e = cudaFuncSetAttribute(k_na_slab, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(smem));
+                                     kSlabBytes);
         if (e == cudaSuccess)
             e = cudaMemsetAsync(s + kPlanes, 0, kNoAllocMaxH * sizeof(unsigned long long), st);
         if (e == cudaSuccess)

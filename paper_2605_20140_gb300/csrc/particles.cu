@@ -1756,10 +1756,18 @@ static int shared_tile_blocks(sipf_ctx* c, size_t smem) {
 
 bool bins_directly(const sipf_ctx* c) { return c->ntiles <= kSharedTiles; }
 
+// Lets these kernels hold up to kSharedTiles words.  The limit belongs to the
+// kernel on the device, not to a context: it is the same whatever the grid, so that
+// another thread's call with a smaller one never lowers it before this one's launch.
+template <class K>
+static cudaError_t allow_shared_tiles(K kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(kSharedTiles * sizeof(int)));
+}
+
 cudaError_t launch_bin(sipf_ctx* c, int b) {
     const size_t smem = static_cast<size_t>(c->ntiles) * sizeof(int);
-    const cudaError_t e = cudaFuncSetAttribute(k_bin, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               static_cast<int>(smem));
+    const cudaError_t e = allow_shared_tiles(k_bin);
     if (e != cudaSuccess) return e;
     k_bin<<<shared_tile_blocks(c, smem), kBinNT, smem, c->stream>>>(
         buf_of(c, b), buf_of(c, b ^ 1), layout_of(c, b ^ 1), static_cast<int>(c->N), c->H,
@@ -1771,8 +1779,7 @@ cudaError_t launch_tile_count(sipf_ctx* c, int b, int* cnt) {
     const int N = static_cast<int>(c->N);
     if (bins_directly(c)) {
         const size_t smem = static_cast<size_t>(c->ntiles) * sizeof(int);
-        const cudaError_t e = cudaFuncSetAttribute(
-            k_tile_count_shared, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        const cudaError_t e = allow_shared_tiles(k_tile_count_shared);
         if (e != cudaSuccess) return e;
         k_tile_count_shared<<<shared_tile_blocks(c, smem), kBinNT, smem, c->stream>>>(
             c->sx[b], c->sy[b], c->sz[b], N, c->H, c->ntiles, cnt);
