@@ -308,6 +308,7 @@ constexpr int kItem = kNT * kPT;          // particles per item
 // 108 us; with kUnitTile = 0 143, since blocks with many thin tiles run long).
 enum Form { kDense, kSparse, kSplit };
 constexpr int kUnit = 2, kUnitTile = 2;
+constexpr int kSplitChunks = 1, kSplitChunks4 = 3;   // most chunks per block of the split form
 constexpr int kBlock = 9 * 9 * 9;         // nodes of a tile's gather block
 constexpr int kSparsePerTile = 256;       // below this mean tile occupancy: sparse form
 
@@ -1616,6 +1617,9 @@ inline Layout layout_of(sipf_ctx* c, int b) {
 }  // namespace
 
 // ---------------------------------------------------------------- launchers
+// Chunks that a run's items can have: a tile ends with one that is not full.
+static int64_t chunks_at_most(const sipf_ctx* c) { return (c->N + kNT - 1) / kNT + c->ntiles; }
+
 int step_grid(sipf_ctx* c) {
     int dev = c->device, nsm = 0, per_sm = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -1629,7 +1633,7 @@ int step_grid(sipf_ctx* c) {
     c->step_blocks_max = g > 0 ? g : 1;
     // no more blocks than items (or, split, chunks) can exist: a small run leaves
     // the rest of the GPU to the runs beside it
-    const int64_t chunks = (c->N + kNT - 1) / kNT + c->ntiles;
+    const int64_t chunks = chunks_at_most(c);
     c->split_blocks = static_cast<int>(chunks < c->step_blocks_max ? chunks : c->step_blocks_max);
     if (g > c->max_items) g = c->max_items;
     return g > 0 ? g : 1;
@@ -1638,17 +1642,22 @@ int step_grid(sipf_ctx* c) {
 cudaError_t launch_step_kernel(sipf_ctx* c, const PushArgs& a, int do_deposit, int do_move) {
     const int b = c->cur;
     // Fewer than kSparsePerTile particles per tile on average: many short items, the
-    // sparse form.  From two chunks per tile on and with fewer full items than
-    // blocks, the split form (32^3 / 2^15: 22.3 -> 18.8 us per step, fourth order
-    // at 64^3 / 2^18 77.5 -> 70.9; with thinner tiles, 72^3 / 2 10^5, it is slower,
-    // 51 against 49 us: two blocks then share a tile that one handles as fast).
+    // sparse form.  From two chunks per tile on, and while each block gets at most
+    // kSplitChunks chunks of all that can exist, the split form.  Split / dense per step,
+    // clouds / evenly spread: trilinear 32^3 / 2^15 0.80 / 0.96, 2^17 0.90 / 0.95; with more
+    // chunks than blocks 32^3 / 192000 1.05 / 1.07, 2^18 1.01 / 1.06, 64^3 / 2^18 1.01 / 1.01, 24^3 /
+    // 648000 1.10 / 1.06, 8^3 / 3 10^5 1.04 / 1.27.  Fourth order, whose chunks take longer: 32^3 /
+    // 2^17 0.81 / 0.92, 64^3 / 2^18 0.93 / 1.01, 48^3 / 324000 0.95 / 0.95; 72^3 / 466560 1.03 / 1.00,
+    // 32^3 / 2^19 1.08 / 1.05.  With thinner tiles it is slower too (72^3 / 2 10^5, 51 against
+    // 49 us: two blocks then share a tile that one handles as fast).
     // Runs beside others (served requests, ensemble members on streams of their
     // own) stay dense: there the SMs' time counts, and split shares enter more
     // tiles (eight requests of 400 steps 77 ms split, 73 dense).
     const int64_t tiles = c->ntiles;
+    const int per_block = c->p.p2g_order == 4 ? kSplitChunks4 : kSplitChunks;
     const int form = c->N < kSparsePerTile * tiles ? kSparse
                    : !c->beside_others && c->N >= 2 * kNT * tiles &&
-                             c->N < static_cast<int64_t>(kItem) * c->step_blocks_max
+                             chunks_at_most(c) <= static_cast<int64_t>(per_block) * c->step_blocks_max
                          ? kSplit : kDense;
     auto pick = [form](auto dense, auto sparse, auto split) {
         return form == kSparse ? sparse : form == kSplit ? split : dense;
