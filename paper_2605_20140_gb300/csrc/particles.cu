@@ -1459,6 +1459,7 @@ __global__ void __launch_bounds__(kStatsNT)
 // below 2^62) rounded to an integer, so the total does not depend on the
 // order in which the particles are stored.
 constexpr int kDiagBlocks = 304;
+constexpr int kThin = 96;          // particles of an item that a warp takes alone
 constexpr int kDiagNT = 256;
 
 __device__ __forceinline__ double dmin(double a, double b) { return a < b ? a : b; }
@@ -1472,16 +1473,37 @@ __global__ void __launch_bounds__(kDiagNT)
     unsigned __int128 mass = 0;
     long long as = 0, amin = LLONG_MAX;
     const int stride = kDiagBlocks * kDiagNT;
-    // particles where they lie in the buckets, item by item (a compact copy of them
-    // first took 58 us at 2^22)
-    const int n = *n_items;
-    for (int q = blockIdx.x; q < n; q += kDiagBlocks) {
-        const int end = items[q].end;
-        for (int i = items[q].beg + threadIdx.x; i < end; i += kDiagNT) {
-            mass += __double2ull_rn(scalbn(exp(src.dl[i]), K));
-            if (!isfinite(src.sx[i]) || !isfinite(src.sy[i]) || !isfinite(src.sz[i])) nf += 1.0;
+    // Particles where they lie in the buckets (a compact copy of them first took 58 us at
+    // 2^22): a block per item, and with many items a warp per thin one, which would leave
+    // most of a block idle (2^20 evenly spread on 256^3, 32 per item: 491 -> 324 us; 4096
+    // items of 16 128 -> 115 us per call; with no more than a few items per block the
+    // warps' longer walks cost more, 16.8 against 10.6 us for 250 items of 66).
+    // The lanes look at 32 items at once for the ones to take.
+    const int n = *n_items, lane = threadIdx.x & 31;
+    const int thin_most = n > 4 * kDiagBlocks ? kThin : 0;
+    auto take = [&](int i) {
+        mass += __double2ull_rn(scalbn(exp(src.dl[i]), K));
+        if (!isfinite(src.sx[i]) || !isfinite(src.sy[i]) || !isfinite(src.sz[i])) nf += 1.0;
+    };
+    auto walk = [&](int first, int step, bool thin, int t, int nt) {
+        for (long long q0 = first; q0 < n; q0 += 32ll * step) {
+            const long long q = q0 + static_cast<long long>(lane) * step;
+            int beg = 0, end = 0;
+            if (q < n) {
+                beg = items[q].beg;
+                end = items[q].end;
+            }
+            unsigned mine = __ballot_sync(kFull, q < n && (end - beg <= thin_most) == thin);
+            for (; mine; mine &= mine - 1) {
+                const int o = __ffs(mine) - 1;
+                const int e = __shfl_sync(kFull, end, o);
+                for (int i = __shfl_sync(kFull, beg, o) + t; i < e; i += nt) take(i);
+            }
         }
-    }
+    };
+    walk(blockIdx.x, kDiagBlocks, false, threadIdx.x, kDiagNT);
+    if (thin_most)
+        walk(blockIdx.x * (kDiagNT / 32) + (threadIdx.x >> 5), stride / 32, true, lane, 32);
     for (int i = blockIdx.x * kDiagNT + threadIdx.x; i < ncell; i += stride) {
         const float a = v[i], b = m[i], c = w[i];
         mv = dmin(mv, a);
