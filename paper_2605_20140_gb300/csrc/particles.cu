@@ -1149,8 +1149,13 @@ __global__ void k_compact(const Item* __restrict__ items, const int* __restrict_
 // particles all lie in its tile, counts the tile's 512 cells in shared memory
 // and adds them to the grid's counters once (particles of the overflow items, and any
 // whose position does not match its bucket, one by one).  Per-particle
-// atomics on a clustered state's cells took 141 us at 128^3 / 2^22, this 18.
+// atomics on a clustered state's cells took 141 us at 128^3 / 2^22, this 18.  An item of at most
+// kFewCells particles counts them one by one all the same: they meet in few words, and the
+// 512 counters of a tile cost more (2^20 evenly spread on 256^3, 32 per item: 43 -> 30 us;
+// the scatter below 85 -> 42).
 constexpr int kCells = kTile * kTile * kTile;
+constexpr int kFewCells = kCells / 4;
+static_assert(kFewCells <= kNT, "a thread for each of a few particles");
 
 __global__ void __launch_bounds__(kNT)
     k_cell_count(const Item* __restrict__ items, const int* __restrict__ n_items, Buf src, int H,
@@ -1158,6 +1163,14 @@ __global__ void __launch_bounds__(kNT)
     __shared__ int hist[kCells];
     if (blockIdx.x >= *n_items) return;
     const Item it = items[blockIdx.x];
+    if (it.end - it.beg <= kFewCells) {
+        const int i = it.beg + static_cast<int>(threadIdx.x);
+        if (i < it.end) {
+            const Cell c = locate_clamped(src.sx[i], src.sy[i], src.sz[i], H);
+            atomicAdd(count + cell_key(c.cx, c.cy, c.cz, H >> 3), 1);
+        }
+        return;
+    }
     for (int l = threadIdx.x; l < kCells; l += kNT) hist[l] = 0;
     __syncthreads();
     for (int i = it.beg + threadIdx.x; i < it.end; i += kNT) {
@@ -1251,6 +1264,17 @@ __global__ void __launch_bounds__(kNT)
     __shared__ int slot[kCells];
     if (blockIdx.x >= *n_items) return;
     const Item it = items[blockIdx.x];
+    if (it.end - it.beg <= kFewCells) {
+        const int i = it.beg + static_cast<int>(threadIdx.x);
+        if (i < it.end) {
+            const Cell c = locate_clamped(src.sx[i], src.sy[i], src.sz[i], H);
+            const uint32_t key = cell_key(c.cx, c.cy, c.cz, H >> 3);
+            const int k = cell_start[key] + atomicAdd(fill + key, 1);
+            keys_tmp[k] = key;
+            ids_tmp[k] = src.id[i];
+        }
+        return;
+    }
     for (int l = threadIdx.x; l < kCells; l += kNT) slot[l] = 0;
     __syncthreads();
     uint32_t keys[kPT];
@@ -1287,26 +1311,34 @@ __global__ void __launch_bounds__(kNT)
 // places brings the runs it touches into shared memory (a dense cell of 128^3 /
 // 2^22 holds hundreds of particles, so they are little more than the block's own
 // places) and each thread reads its run there, the lanes of a warp mostly the same
-// one; runs that do not fit are read from global memory.  A tie counts for the
+// one; runs that do not fit, and blocks of short runs (evenly spread 17 -> 15 us at 2^20), are
+// read from global memory.  A tie counts for the
 // places before j only, so the loop is split there.  225 -> 194 us at 128^3 / 2^22
 // (ncu), bound by the 10^9 comparisons.
 constexpr int kRankNT = 256;
 constexpr int kRankIds = 2560;
+constexpr int kShortRun = 16;
 
 __global__ void __launch_bounds__(kRankNT)
     k_canon_rank(const uint32_t* __restrict__ keys_tmp, const uint32_t* __restrict__ ids_tmp, int N,
                  const int* __restrict__ cell_start, uint32_t* __restrict__ out) {
     __shared__ uint32_t ids[kRankIds];
+    __shared__ int range[2];
     const int j0 = blockIdx.x * kRankNT, j1 = min(j0 + kRankNT, N) - 1;
-    const int lo = cell_start[keys_tmp[j0]], hi = cell_start[keys_tmp[j1] + 1];
-    const bool held = hi - lo <= kRankIds;
-    if (held)
-        for (int t = threadIdx.x; t < hi - lo; t += kRankNT) ids[t] = ids_tmp[lo + t];
-    __syncthreads();
-    const int j = j0 + static_cast<int>(threadIdx.x);
-    if (j > j1) return;
+    const int j = min(j0 + static_cast<int>(threadIdx.x), j1);
     const uint32_t key = keys_tmp[j];
     const int b = cell_start[key], e = cell_start[key + 1];
+    if (threadIdx.x == 0) range[0] = b;
+    if (j == j1) range[1] = e;
+    // only short runs in the block: read in place, their ids are still close by
+    const bool some_long = __syncthreads_or(e - b > kShortRun);
+    const int lo = range[0], hi = range[1];
+    const bool held = some_long && hi - lo <= kRankIds;
+    if (held) {
+        for (int t = threadIdx.x; t < hi - lo; t += kRankNT) ids[t] = ids_tmp[lo + t];
+        __syncthreads();
+    }
+    if (j0 + static_cast<int>(threadIdx.x) > j1) return;
     int rank = 0;
     uint32_t me;
     if (held) {
