@@ -134,7 +134,7 @@ int sipf_create(const sipf_grid* grid, int64_t N, const sipf_params* params,
  * (H^3 floats each).  grad v is computed from v by the spectral derivative
  * (Eq. gradv) and the particles are binned by cell.  Resets the step counter
  * and the time to 0.  Errors: SIPF_EINVAL (NULL pointer, bad `where`, a
- * negative or non-finite mass), SIPF_ECUDA. */
+ * negative or non-finite mass), SIPF_ENOMEM (host memory), SIPF_ECUDA. */
 int sipf_set_state(sipf_ctx* ctx, const float* x, const double* mass, const uint32_t* id,
                    const float* v, const float* m, const float* w, int where);
 

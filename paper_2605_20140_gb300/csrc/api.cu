@@ -226,10 +226,14 @@ void free_all(sipf_ctx* c) {
             cudaFree(q);
     }
     if (c->rs_scratch) cudaFree(c->rs_scratch);
-    if (c->hstage) cudaFreeHost(c->hstage);
+    c->hstage.release([](void* q) { cudaFreeHost(q); });
 }
 
-constexpr size_t kStage = size_t{1} << 16;   // masses per half of the pinned staging buffer
+constexpr size_t kStage = size_t{1} << 16;   // masses per half of the host staging buffer
+// Pinning that buffer takes 0.13 ms, which a first call pays back from kPinFrom masses on (2^14
+// unequal masses 270 us without, 310 with; 7 10^5 1.30 and 1.09 ms), and a second call with
+// two halves or more (2^18: 484 us unpinned, 464 pinned).
+constexpr size_t kPinFrom = 8 * kStage;
 
 int copy_in(sipf_ctx* c, void* dst, const void* src, size_t bytes, int where) {
     const cudaMemcpyKind k = where == SIPF_DEVICE ? cudaMemcpyDeviceToDevice
@@ -742,20 +746,22 @@ int sipf_set_state(sipf_ctx* c, const float* x, const double* mass, const uint32
         if (where == SIPF_HOST) {
             ok = add(mass, N);
         } else {
-            // through two halves of a pinned buffer of the context, so that one half
-            // is summed while the other is copied (2^20 masses: 0.3 ms less than one pageable copy of all of
-            // them into fresh memory)
-            if (!c->hstage && cudaMallocHost(&c->hstage, 2 * kStage * sizeof(double)) != cudaSuccess) {
-                cudaGetLastError();
-                c->hstage = nullptr;
-                return fail(c, SIPF_ENOMEM, "pinned staging buffer");
-            }
+            // through two halves of a buffer of the context, so that, pinned, one half
+            // is summed while the other is copied (2^20 masses: 0.3 ms less than one pageable
+            // copy of all of them into fresh memory)
+            auto pin = [](void** q, size_t bytes) {
+                const bool ok = cudaMallocHost(q, bytes) == cudaSuccess;
+                if (!ok) cudaGetLastError();
+                return ok;
+            };
+            if (!c->hstage.get(std::min(N, 2 * kStage), N >= kPinFrom, N >= 2 * kStage, pin))
+                return fail(c, SIPF_ENOMEM, "host staging buffer");
             const cudaEvent_t ev[2] = {c->ev_fork, c->ev_join};   // idle outside a step
             const size_t parts = (N + kStage - 1) / kStage;
             for (size_t k = 0; k <= parts && ok; ++k) {
                 if (k < parts) {
                     const size_t o = k * kStage, n = std::min(kStage, N - o);
-                    SIPF_CUDA(c, cudaMemcpyAsync(c->hstage + (k & 1) * kStage, mass + o,
+                    SIPF_CUDA(c, cudaMemcpyAsync(c->hstage.p + (k & 1) * kStage, mass + o,
                                                  n * sizeof(double), cudaMemcpyDeviceToHost,
                                                  c->stream));
                     SIPF_CUDA(c, cudaEventRecord(ev[k & 1], c->stream));
@@ -763,7 +769,7 @@ int sipf_set_state(sipf_ctx* c, const float* x, const double* mass, const uint32
                 if (k > 0) {
                     const size_t o = (k - 1) * kStage, n = std::min(kStage, N - o);
                     SIPF_CUDA(c, cudaEventSynchronize(ev[(k - 1) & 1]));
-                    ok = add(c->hstage + ((k - 1) & 1) * kStage, n);
+                    ok = add(c->hstage.p + ((k - 1) & 1) * kStage, n);
                 }
             }
             if (!ok) cudaStreamSynchronize(c->stream);
@@ -777,7 +783,7 @@ int sipf_set_state(sipf_ctx* c, const float* x, const double* mass, const uint32
     c->time = 0.0;
     // wrap into buffer 1 (unordered), then bin into buffer 0.  Host input is
     // staged in buffer 0 first (free until the binning; each of its arrays
-    // has room for N values), so the call allocates nothing.
+    // has room for N values), so the call allocates no device memory.
     const float* px = x;
     const float* py = x + N;
     const float* pz = x + 2 * N;

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "../../include/sipf.h"
+#include "host_stage.h"
 
 namespace sipf {
 
@@ -318,7 +319,7 @@ struct sipf_ctx {
     float* voff = nullptr;           // device scalar: offset subtracted from v before its FFT
     int kxp = 0;
 
-    double* hstage = nullptr;        // pinned staging of unequal masses (allocated on first use)
+    sipf::HostStage hstage;          // staging of unequal masses (allocated on first use)
     void* rs_scratch = nullptr;      // residual resampling work space (allocated on first use)
     size_t rs_bytes = 0;
 
