@@ -19,6 +19,7 @@
 #include <mutex>
 
 #include "sipf_internal.cuh"
+#include "slab_shares.h"
 
 namespace {
 
@@ -193,13 +194,6 @@ __global__ void __launch_bounds__(kNaNT)
 constexpr int kSlabNT = 512;
 constexpr int kScan = 4;        // z read per thread and round
 
-constexpr int kSlabBytes = 200 * 1024;   // a slab's node sums at most, eight bytes each
-
-__host__ __device__ inline int na_slab_planes(int H) {   // planes per slab, one more is held
-    const int p = kSlabBytes / (H * H * 8) - 1;
-    return p < H ? p : H;
-}
-
 __global__ void __launch_bounds__(kSlabNT)
     k_na_slab(const float* __restrict__ x, const double* __restrict__ mass, int64_t N, int H,
               float o0, float o1, float o2, float h, int parts, unsigned long long* s) {
@@ -207,7 +201,7 @@ __global__ void __launch_bounds__(kSlabNT)
     __shared__ int mine[3];                       // slab, part of it, its parts
     __shared__ int queue[kSlabNT / 32][32 * (kScan + 1)];
     sipf::pdl_trigger();
-    const int P = na_slab_planes(H), slabs = (H + P - 1) / P, plane = H * H;
+    const int P = sipf::slab_planes(H), slabs = (H + P - 1) / P, plane = H * H;
     const int nodes = (P + 1) * plane;
     uint32_t* lo = sm;
     uint32_t* hi = sm + nodes;
@@ -228,7 +222,7 @@ __global__ void __launch_bounds__(kSlabNT)
     if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = mx;
     if (threadIdx.x == 0) {
         // blocks per slab: in proportion to its particles plus the reading of all z
-        // (about a 24th of a particle each), at least one
+        // (about a 24th of a particle each), at least one (the grid has that many)
         double all = 0.0;
         for (int k = 0; k < H; ++k) all += static_cast<double>(s[kPlanes + k]);
         const double scan = static_cast<double>(N) / 24.0, total = all + scan * slabs;
@@ -389,19 +383,20 @@ extern "C" int sipf_deposit_noalloc(const sipf_grid* grid, const float* x, const
         e = cudaGetDevice(&dev);
         if (e == cudaSuccess)
             e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        const size_t smem = static_cast<size_t>(na_slab_planes(H) + 1) * H * H * 2 * sizeof(uint32_t);
+        const size_t smem =
+            static_cast<size_t>(sipf::slab_planes(H) + 1) * H * H * 2 * sizeof(uint32_t);
         if (e == cudaSuccess)
             // the limit belongs to the kernel, not to this call: the same for every H
             e = cudaFuncSetAttribute(k_na_slab, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     kSlabBytes);
+                                     sipf::kSlabBytes);
         if (e == cudaSuccess)
             e = cudaMemsetAsync(s + kPlanes, 0, kNoAllocMaxH * sizeof(unsigned long long), st);
         if (e == cudaSuccess)
             e = sipf::launch_pdl(k_na_begin, dim3(parts), dim3(kNaNT), 0, st, mass, N, nodes,
                                  x + 2 * N, H, o2, hf, s);
         if (e == cudaSuccess)
-            e = sipf::launch_pdl(k_na_slab, dim3(nsm), dim3(kSlabNT), smem, st, x, mass, N, H, o0,
-                                 o1, o2, hf, parts, s);
+            e = sipf::launch_pdl(k_na_slab, dim3(sipf::slab_grid(nsm, H)), dim3(kSlabNT), smem, st,
+                                 x, mass, N, H, o0, o1, o2, hf, parts, s);
     }
     if (e == cudaSuccess)
         e = sipf::launch_pdl(k_na_finish, dim3(nblocks), dim3(kNaNT), 0, st,
