@@ -683,6 +683,7 @@ int create_in_pool(const sipf_grid* grid, int64_t N, const sipf_params* params,
     sipf_tuning tuned;
     if (lookup_tuning(c->H, N, &tuned)) apply_tuning(c, tuned);
     c->step_blocks = step_grid(c);
+    c->plan_blocks = plan_grid(c);
     if (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess) {

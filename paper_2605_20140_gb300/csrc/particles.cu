@@ -19,14 +19,15 @@
 // and needs no float atomics), gathers grad v and w at X^(n-1), draws the Philox normals,
 // pushes, updates the log-mass, and writes the particle into its new tile's
 // bucket straight from registers: the lanes of a warp bound for the same
-// tile reserve consecutive slots with one global atomic.  A one-block plan
-// kernel then builds the next step's items and the next bucket layout from
-// the counts.
+// tile reserve consecutive slots with one global atomic.  A plan kernel (one
+// block, on large grids a cluster of eight) then builds the next step's items and
+// the next bucket layout from the counts.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 
+#include "plan_shape.h"
 #include "sipf_internal.cuh"
 
 namespace sipf {
@@ -769,10 +770,7 @@ __global__ void __launch_bounds__(kNT, DepBlock<ORDER>::MIN_BLOCKS)
 }
 
 // ------------------------------------------------------------------ planning
-// Block-wide exclusive scan (one value per thread) of kPlanNT threads.
-constexpr int kPlanNT = 512;
-constexpr int kPlanCluster = 8;   // blocks of the plan kernel on large grids
-
+// Block-wide exclusive scan, one value per thread (up to 1024).
 __device__ __forceinline__ int block_exclusive_scan(int v, int* smem, int* total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int incl = v;
@@ -1729,24 +1727,38 @@ cudaError_t launch_step_kernel(sipf_ctx* c, const PushArgs& a, int do_deposit, i
                       c->status);
 }
 
-// Items of buffer `b` and, with next_layout, the layout of b ^ 1.  One block of
-// 32 warps up to 1024 tiles (H = 80), a strip or less per warp; a cluster of
-// eight beyond.
+static cudaLaunchConfig_t plan_config(int blocks, cudaLaunchAttribute* attr) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(kPlanNT);
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = blocks;
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = blocks > 1 ? 1 : 0;
+    return cfg;
+}
+
+int plan_grid(sipf_ctx* c) {
+    if (plan_blocks(c->ntiles, 1) == 1) return 1;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = plan_config(kPlanCluster, &attr);
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, k_plan<kPlanCluster>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        clusters = 0;
+    }
+    return plan_blocks(c->ntiles, clusters);
+}
+
+// Items of buffer `b` and, with next_layout, the layout of b ^ 1.
 cudaError_t launch_plan(sipf_ctx* c, int b, int next_layout, cudaStream_t s, double dt) {
     const int o = b ^ 1;
-    const bool cluster = c->ntiles > 2 * kPlanNT;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(cluster ? kPlanCluster : 1);
-    cfg.blockDim = dim3(kPlanNT);
+    cudaLaunchAttribute attr;
+    cudaLaunchConfig_t cfg = plan_config(c->plan_blocks, &attr);
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kPlanCluster;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = cluster ? 1 : 0;
     return cudaLaunchKernelEx(
-        &cfg, cluster ? k_plan<kPlanCluster> : k_plan<1>, c->ntiles, c->H / 8,
+        &cfg, c->plan_blocks > 1 ? k_plan<kPlanCluster> : k_plan<1>, c->ntiles, c->H / 8,
         static_cast<const int*>(c->cnt[b]), static_cast<const int*>(c->cap[b]),
         static_cast<const int*>(c->bstart[b]), static_cast<const int*>(c->ovf[b]), c->ovf_base,
         c->items, c->n_items, next_layout ? c->bstart[o] : nullptr,

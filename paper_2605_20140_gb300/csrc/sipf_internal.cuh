@@ -294,6 +294,7 @@ struct sipf_ctx {
     int step_blocks = 0;                 // blocks of the particle step
     int step_blocks_max = 1;             // as many as fit on the GPU (or the tuning allows)
     int split_blocks = 1;                // of its split form
+    int plan_blocks = 1;                 // of the plan kernel
 
     // per-cell histogram (sipf_cell_start)
     int32_t* count = nullptr;        // H^3
@@ -358,6 +359,7 @@ namespace sipf {
 // ---------------------------------------------------------------- launchers
 // particles.cu
 int step_grid(sipf_ctx* c);
+int plan_grid(sipf_ctx* c);
 int item_size();
 size_t diag_scratch_doubles();
 size_t diag_scratch_ll();
