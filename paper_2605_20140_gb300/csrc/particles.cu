@@ -1446,6 +1446,7 @@ __global__ void k_set_w(const float* __restrict__ w, int n, float* __restrict__ 
 // memory speed.
 constexpr int kStatsBlocks = 304;
 constexpr int kStatsNT = 256;
+static_assert(alignof(StateStats) <= alignof(double), "kept in an array of doubles");
 
 __global__ void __launch_bounds__(kStatsNT)
     k_state_stats(const double* __restrict__ mass, int N, const float* __restrict__ v, int n,
@@ -2005,7 +2006,12 @@ cudaError_t launch_normals(const uint32_t* ids, int64_t N, uint32_t n, uint64_t 
     return cudaGetLastError();
 }
 
-size_t diag_scratch_doubles() { return static_cast<size_t>(kDiagBlocks) * 5; }
+// The buffer of the diagnostics' partial sums, which also takes a new state's statistics.
+size_t diag_scratch_doubles() {
+    constexpr size_t diag = kDiagBlocks * 5;
+    constexpr size_t stats = (kStatsBlocks * sizeof(StateStats) + sizeof(double) - 1) / sizeof(double);
+    return diag > stats ? diag : stats;
+}
 size_t diag_scratch_ll() { return static_cast<size_t>(kDiagBlocks) * 4; }
 int scan_tiles(int n) { return (n + kScanTile - 1) / kScanTile; }
 int item_size() { return kItem; }
