@@ -4,6 +4,7 @@
 // them has to give the same bits.
 #pragma once
 
+#include <float.h>
 #include <math.h>
 #include <stdint.h>
 
@@ -25,10 +26,12 @@ inline double ordered_sum_of_equal(double m, int64_t n) {
             const double end = ldexp(1.0, ilogb(acc) + 1);   // acc lies in [end/2, end)
             const double d = next - acc;                      // exact: both are multiples of u
             // m - d is exact (|m - d| <= u/2, both multiples of m's spacing or finer)
-            const bool tie = fabs(m - d) == 0.5 * (end * 0x1p-53);
+            const bool tie = fabs(m - d) == 0.5 * ldexp(1.0, ilogb(acc) - 52);
             if (!tie && d > 0.0 && next < end) {
-                // steps that certainly stay below end (m <= d + u/2 < 2 d + u)
-                int64_t t = static_cast<int64_t>((end - next) / d) - 3;
+                // steps that certainly stay below end (m <= d + u/2 < 2 d + u), and below
+                // the largest number in the topmost binade, whose end is not one
+                const double room = (isfinite(end) ? end : DBL_MAX) - next;
+                int64_t t = static_cast<int64_t>(room / d) - 3;
                 if (t > n) t = n;
                 if (t > 0) {
                     acc = next + static_cast<double>(t) * d;
