@@ -835,6 +835,10 @@ int sipf_set_state(sipf_ctx* c, const float* x, const double* mass, const uint32
         if (r == SIPF_OK) r = copy_in(c, c->m, m, H3 * sizeof(float), where);
         if (r == SIPF_OK) r = copy_in(c, c->w, w, H3 * sizeof(float), where);
     }
+    // A step that failed between its launches may have left a deposit.  The forward plane
+    // pass below clears it, the per-axis one only with m and w.
+    if (e == cudaSuccess && r == SIPF_OK && (c->H > 128 || c->radix_plan == 2))
+        e = cudaMemsetAsync(c->acc, 0, H3 * sizeof(long long), c->stream);
     if (e == cudaSuccess && r == SIPF_OK) r = bin_initial(c);
     if (e == cudaSuccess && r == SIPF_OK) {
         // w^(0) into the gather array; grad v^(0) from the DFT of v^(0) (tau = 0)
