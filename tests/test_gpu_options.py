@@ -17,6 +17,12 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
+@pytest.fixture(autouse=True)
+def _needs_gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
 def _run(wl, plan, steps):
     stream = torch.cuda.Stream()
     with sipf.Simulation(wl.H, wl.L, wl.origin, wl.N, wl.params,
