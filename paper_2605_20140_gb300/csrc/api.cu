@@ -365,6 +365,7 @@ int bin_initial(sipf_ctx* c) { return bin_from(c, 1); }
 // Deposit the current particles into the accumulator (Alg. 1).
 int deposit_current(sipf_ctx* c) {
     const PushArgs a = push_args(c, 0.0, 0);
+    c->deposited = true;
     SIPF_CUDA(c, launch_step_kernel(c, a, 1, 0));
     return SIPF_OK;
 }
@@ -405,6 +406,7 @@ int enqueue_step(sipf_ctx* c, double dt) {
     const PushArgs a = push_args(c, dt, 1);
     const SpectralArgs sa = spectral_args(c, dt, 1);
     SIPF_CUDA(c, prof_mark(c, 0));
+    c->deposited = true;
     SIPF_CUDA(c, launch_step_kernel(c, a, 1, 1));
     SIPF_CUDA(c, prof_mark(c, 1));
     // the plan of the next step's items, layout and scalars needs only the
@@ -419,6 +421,7 @@ int enqueue_step(sipf_ctx* c, double dt) {
         SIPF_CUDA(c, launch_spectral_pass(c, sa, pass));
         SIPF_CUDA(c, prof_mark(c, 2 + pass));
     }
+    c->deposited = false;   // cleared by the forward pass
     SIPF_CUDA(c, cudaStreamWaitEvent(c->stream, c->ev_join, 0));
     if (c->prof_on && c->prof_steps < kProfMaxSteps) c->prof_steps += 1;
     advance_host(c, dt);
@@ -835,10 +838,10 @@ int sipf_set_state(sipf_ctx* c, const float* x, const double* mass, const uint32
         if (r == SIPF_OK) r = copy_in(c, c->m, m, H3 * sizeof(float), where);
         if (r == SIPF_OK) r = copy_in(c, c->w, w, H3 * sizeof(float), where);
     }
-    // A step that failed between its launches may have left a deposit.  The forward plane
-    // pass below clears it, the per-axis one only with m and w.
-    if (e == cudaSuccess && r == SIPF_OK && (c->H > 128 || c->radix_plan == 2))
+    // what a call that failed after its deposit left in the accumulator
+    if (e == cudaSuccess && r == SIPF_OK && c->deposited)
         e = cudaMemsetAsync(c->acc, 0, H3 * sizeof(long long), c->stream);
+    if (e == cudaSuccess && r == SIPF_OK) c->deposited = false;
     if (e == cudaSuccess && r == SIPF_OK) r = bin_initial(c);
     if (e == cudaSuccess && r == SIPF_OK) {
         // w^(0) into the gather array; grad v^(0) from the DFT of v^(0) (tau = 0)
@@ -894,8 +897,10 @@ int sipf_fields(sipf_ctx* c, uint32_t mask, float* dst, int where) {
             if (r != SIPF_OK) return r;
             if (where == SIPF_DEVICE) {
                 SIPF_CUDA(c, launch_acc_to_float(c, dst + off, acc_to_u(c)));
+                c->deposited = false;
             } else {
                 cudaError_t e = launch_acc_to_float(c, tmp, acc_to_u(c));
+                if (e == cudaSuccess) c->deposited = false;
                 if (e == cudaSuccess)
                     e = cudaMemcpyAsync(dst + off, tmp, H3 * sizeof(float), cudaMemcpyDeviceToHost,
                                         c->stream);
@@ -1036,6 +1041,7 @@ int sipf_diagnostics(sipf_ctx* c, sipf_diag* out) {
     SIPF_CUDA(c, launch_diagnostics(c, acc_to_u_d(c)));
     const size_t H3 = static_cast<size_t>(c->H) * c->H * c->H;
     SIPF_CUDA(c, cudaMemsetAsync(c->acc, 0, H3 * sizeof(long long), c->stream));
+    c->deposited = false;
     double h[8];
     SIPF_CUDA(c, cudaMemcpyAsync(h, c->diag_out, 7 * sizeof(double), cudaMemcpyDeviceToHost,
                                  c->stream));
@@ -1341,6 +1347,7 @@ int enqueue_batched_step(sipf_ensemble* e, const double* dt, const RunDesc* d_ru
         e->last_error = std::string(where) + ": " + cudaGetErrorString(err);
         return SIPF_ECUDA;
     };
+    for (sipf_ctx* c : e->members) c->deposited = true;
     int r = cuda(launch_step_multi(d_runs, n, parity, e->main), "batched particle step");
     if (r == SIPF_OK) r = cuda(cudaEventRecord(e->ev_fork, e->main), "cudaEventRecord");
     if (r == SIPF_OK) r = cuda(cudaStreamWaitEvent(e->side, e->ev_fork, 0), "cudaStreamWaitEvent");
@@ -1386,7 +1393,10 @@ int enqueue_batched_step(sipf_ensemble* e, const double* dt, const RunDesc* d_ru
         if (r == SIPF_OK) r = cuda(cudaStreamWaitEvent(e->main, ev, 0), "cudaStreamWaitEvent");
     if (r == SIPF_OK) r = cuda(cudaStreamWaitEvent(e->main, e->ev_join, 0), "cudaStreamWaitEvent");
     if (r != SIPF_OK) return r;
-    for (int i = 0; i < n; ++i) advance_host(e->members[i], dt[i]);
+    for (int i = 0; i < n; ++i) {
+        advance_host(e->members[i], dt[i]);
+        e->members[i]->deposited = false;
+    }
     return SIPF_OK;
 }
 

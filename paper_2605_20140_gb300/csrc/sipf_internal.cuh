@@ -303,6 +303,7 @@ struct sipf_ctx {
 
     // grid
     long long* acc = nullptr;        // H^3 fixed-point deposit accumulator, zero between steps
+    bool deposited = false;          // a call in progress (or failed) has deposited into it
     float* us = nullptr;             // K_sigma * u_bar, the m source (sigma > 0 only)
     float* ksig = nullptr;           // [H] 1D smoothing multiplier exp(-sigma k_j^2 / 2) / H
     float* v = nullptr;
