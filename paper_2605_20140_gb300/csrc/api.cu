@@ -193,7 +193,7 @@ size_t ctx_device_bytes(int H, int64_t N, bool filter, bool smoothing) {
     const size_t S = static_cast<size_t>(z.buf_slots);
     size_t b = 2 * (S * (3 * sizeof(float) + sizeof(double) + sizeof(uint32_t)) +
                     3 * static_cast<size_t>(z.ntiles) * sizeof(int) + sizeof(int));
-    b += static_cast<size_t>(z.max_items) * sizeof(Item) + 3 * sizeof(int);
+    b += static_cast<size_t>(z.max_items) * sizeof(Item) + 2 * sizeof(int);
     b += z.H3 * sizeof(int32_t) + (z.H3 + 1) * sizeof(int32_t) +
          (static_cast<size_t>(scan_tiles(static_cast<int>(z.H3))) + 1) * sizeof(int32_t);
     b += z.H3 * sizeof(long long) + 3 * z.H3 * sizeof(float) + 4 * z.H3 * sizeof(float);
@@ -213,7 +213,7 @@ void free_all(sipf_ctx* c) {
     void* ptrs[] = {c->sx[0], c->sx[1], c->sy[0], c->sy[1], c->sz[0], c->sz[1], c->dl[0],
                     c->dl[1], c->id[0], c->id[1], c->bstart[0], c->bstart[1], c->cap[0],
                     c->cap[1], c->cnt[0], c->cnt[1], c->ovf[0], c->ovf[1], c->items, c->n_items,
-                    c->work, c->count, c->cell_start, c->scan_tmp, c->acc, c->v, c->m, c->w,
+                    c->count, c->cell_start, c->scan_tmp, c->acc, c->v, c->m, c->w,
                     c->G, c->specM, c->specW, c->specV, c->specB, c->specA, c->specDx,
                     c->specDy, c->twiddle,
                     c->status, c->diag_tmp, c->diag_out, c->diag_ll, c->voff,
@@ -631,7 +631,7 @@ int create_in_pool(const sipf_grid* grid, int64_t N, const sipf_params* params,
              da(&c->cnt[b], c->ntiles) == cudaSuccess && da(&c->ovf[b], 1) == cudaSuccess;
     }
     ok = ok && da(&c->items, static_cast<size_t>(c->max_items)) == cudaSuccess &&
-         da(&c->n_items, 2) == cudaSuccess && da(&c->work, 1) == cudaSuccess &&
+         da(&c->n_items, 2) == cudaSuccess &&
          da(&c->count, H3) == cudaSuccess && da(&c->cell_start, H3 + 1) == cudaSuccess &&
          da(&c->scan_tmp, static_cast<size_t>(scan_tiles(static_cast<int>(H3))) + 1) == cudaSuccess &&
          da(&c->acc, H3) == cudaSuccess && da(&c->v, H3) == cudaSuccess &&

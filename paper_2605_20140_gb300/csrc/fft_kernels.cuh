@@ -61,7 +61,11 @@ template <> struct LineCfg<432> { static constexpr int NT = 384, NTX = 224; };
 template <> struct LineCfg<512> { static constexpr int NT = 512, NTX = 256; };
 
 // Blocks per SM the registers of the row and line passes are set for: 64 registers a
-// thread, or 56 where that lets a third block of 384 threads share the SM.
+// thread, 56 at 288 and 384, where a third block of 384 threads then shares the SM.  The rule
+// stands as measured at these sizes; 432 has 384 threads too, but its z pass wants 80 registers
+// (two blocks, 88 bytes spilled in plan 0) and has not been measured with fewer.  The caps
+// spill 96 to 120 bytes in k_rows_forward at 144 (plan 0), 192, 288 and 384, 36 at 256 and
+// in k_lines_z at 288.
 template <int H> constexpr int line_blocks() {
     return 65536 / ((H == 288 || H == 384 ? 56 : 64) * LineCfg<H>::NT);
 }
@@ -565,7 +569,7 @@ __global__ void __launch_bounds__(LineCfg<H>::NT)
                   : family == 2 ? (SIGN < 0 ? R.specV : R.specB)
                   : family == 3 ? R.specDx : R.specDy) + base;
     const float ks = a.two_pi_over_L;
-    one_way<H, V, kCols, NT, SIGN, false, false>(
+    one_way<H, V, kCols, NT, SIGN>(
         buf, tw, Strided<1, kCols>{},
         [=](int, int y) {
             if (!in) return make_float2(0.f, 0.f);

@@ -216,11 +216,6 @@ __device__ __forceinline__ void stage(float2* buf, const float2* tw) {
     stage_at<L, R, NS, NTRANS, NT, SIGN>(buf, tw, Strided<TS, ES>{});
 }
 
-template <int L, int R, int NS, int NTRANS, int ES, int TS, int NT, int SIGN, class Sink>
-__device__ __forceinline__ void stage_sink(const float2* buf, const float2* tw, Sink sink) {
-    stage_sink_at<L, R, NS, NTRANS, NT, SIGN>(buf, tw, Strided<TS, ES>{}, sink);
-}
-
 // First Stockham stage (NS = 1) with inputs from a loader: element j of
 // transform t is load(t, j).  All loads precede all writes (a block barrier
 // in between), so the loader may read the memory `out` overwrites.
@@ -328,11 +323,6 @@ __device__ __forceinline__ void fft_rest_at(float2* buf, const float2* tw, At at
 template <int L, int V, int NTRANS, int ES, int TS, int NT, int SIGN>
 __device__ __forceinline__ void fft_rest(float2* buf, const float2* tw) {
     fft_rest_at<L, V, NTRANS, NT, SIGN>(buf, tw, Strided<TS, ES>{});
-}
-
-template <int L, int V, int NTRANS, int ES, int TS, int NT, int SIGN, class Sink>
-__device__ __forceinline__ void fft_rest_sink(float2* buf, const float2* tw, Sink sink) {
-    fft_rest_sink_at<L, V, NTRANS, NT, SIGN>(buf, tw, Strided<TS, ES>{}, sink);
 }
 
 // Batched length-L FFT along one axis, in place (radix plan V).
@@ -504,10 +494,8 @@ __device__ __forceinline__ void round_trip(float2* buf, const float2* tw, At at,
     }
 }
 
-// One DFT of NTRANS lines from load to store through buf; JF1 and JFL: the
-// lane order of the first and of the last stage (see stage_ls).
-template <int L, int V, int NTRANS, int NT, int SIGN, bool JF1, bool JFL, class At, class Load,
-          class Store>
+// One DFT of NTRANS lines from load to store through buf.
+template <int L, int V, int NTRANS, int NT, int SIGN, class At, class Load, class Store>
 __device__ __forceinline__ void one_way(float2* buf, const float2* tw, At at, Load load,
                                         Store store) {
     using P = Radix<L, V>;
@@ -515,7 +503,7 @@ __device__ __forceinline__ void one_way(float2* buf, const float2* tw, At at, Lo
     constexpr int RL = R4 > 1 ? R4 : R3 > 1 ? R3 : R2;
     auto sload = [=](int t, int p) { return buf[at(t, p)]; };
     auto sstore = [=](int t, int p, float2 v) { buf[at(t, p)] = v; };
-    stage_ls<L, R1, 1, NTRANS, NT, SIGN, JF1, false>(tw, load, sstore);
+    stage_ls<L, R1, 1, NTRANS, NT, SIGN, false, false>(tw, load, sstore);
     __syncthreads();
     if constexpr (R3 > 1) {
         stage_ls<L, R2, R1, NTRANS, NT, SIGN, false, true>(tw, sload, sstore);
@@ -525,7 +513,7 @@ __device__ __forceinline__ void one_way(float2* buf, const float2* tw, At at, Lo
         stage_ls<L, R3, R1 * R2, NTRANS, NT, SIGN, false, true>(tw, sload, sstore);
         __syncthreads();
     }
-    stage_ls<L, RL, L / RL, NTRANS, NT, SIGN, JFL, false>(tw, sload, store);
+    stage_ls<L, RL, L / RL, NTRANS, NT, SIGN, false, false>(tw, sload, store);
 }
 
 }  // namespace fftk

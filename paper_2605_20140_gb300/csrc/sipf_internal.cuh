@@ -289,7 +289,6 @@ struct sipf_ctx {
     int* ovf[2] = {nullptr, nullptr};    // particles in the overflow region
     sipf::Item* items = nullptr;         // items of the current buffer
     int* n_items = nullptr;              // [2]: items, work units
-    int* work = nullptr;                 // work counter of the persistent step kernel
     int max_items = 0;
     int step_blocks = 0;                 // blocks of the particle step
     int step_blocks_max = 1;             // as many as fit on the GPU (or the tuning allows)
